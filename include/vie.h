@@ -58,8 +58,9 @@ enum {
                                  5-smooth size >= 2n - 1) */
   VIE_PLAN_AUTOTUNE = 2       /* time complex64 operator applications for the
                                  three smallest 5-smooth sizes >= 2n - 1 per axis
-                                 and the x-pass variants (four-step with 2 or 4
-                                 lines per block, three-factor with 1 or 2)
+                                 and the x-pass variants compiled for lines of
+                                 600 values (four-step and three-factor, five
+                                 lines per block)
                                  of the forward and the inverse pass, keep the
                                  fastest (any M >= 2n - 1 embeds the operator
                                  exactly); ignored with VIE_PLAN_CIRC_2N */
@@ -76,12 +77,11 @@ typedef struct {
   int x_lines_per_block;      /* forward x pass chosen by the tuner: > 0 four-step
                                  register FFT with that many lines per block,
                                  < 0 three-factor register FFT with -value lines
-                                 per block, 0 the default (three-factor where
-                                 compiled for Mx, else four-step; five lines
-                                 per block in complex64 when that makes one
-                                 block per SM, e.g. nx = 600 with 759 lines) */
-  int x_lines_per_block_inverse; /* the same for the inverse x pass (its default:
-                                    four-step where compiled for Mx) */
+                                 per block, 0 the default (five lines per block
+                                 of the kernels compiled for nx = 600 in
+                                 complex64 when that makes one block per SM,
+                                 else the kernel for any length) */
+  int x_lines_per_block_inverse; /* the same for the inverse x pass */
 } vie_plan_info;
 
 /* Graded absorber of Sec. 4.1-4.2: eps'' = eps2_max * u^degree with

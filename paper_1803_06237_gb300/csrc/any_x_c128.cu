@@ -1,0 +1,7 @@
+// The x passes of any_x.cuh on complex128 vectors (a file of its own: it compiles beside the others).
+#include "any_x.cuh"
+
+namespace vie {
+template vie_status launch_x_any<double2>(bool, const PassPtrs<double2>&, int, int, int, int, int, const double2*, int,
+                                      cudaStream_t, int, bool*);
+}  // namespace vie

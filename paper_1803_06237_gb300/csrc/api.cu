@@ -407,17 +407,14 @@ static vie_status autotune(vie_plan* p, cudaStream_t s) {
     for (int cy = 0; cy < 3; ++cy)
       for (int cz = 0; cz < 3; ++cz) {
         set_config(cx, cy, cz);
-        int l1 = 0, l2 = 0, a1 = 0, a2 = 0, a3 = 0;
-        x4_factors(p->m[0], &l1, &l2);
-        x3_factors(p->m[0], &a1, &a2, &a3);
-        // x-pass variants: four-step with 2 or 4 lines per block, three-factor
-        // with 1 or 2 (negative codes), and 5 of either where five-line blocks
-        // fill the SMs once, for the forward and the inverse pass
-        std::vector<int> modes;
-        const bool five = x_lines_five((long)NL, 1) && p->n[0] == 600;
-        if (l1) { modes.push_back(2); modes.push_back(4); if (five) modes.push_back(5); }
-        if (a1) { modes.push_back(-1); modes.push_back(-2); if (five) modes.push_back(-5); }
-        if (modes.empty()) modes.push_back(0);
+        // x-pass variants: the default, and the compiled four-step (5) and
+        // three-factor (-5) kernels of five lines per block where they fill
+        // the SMs once, for the forward and the inverse pass
+        std::vector<int> modes(1, 0);
+        if (x_lines_five((long)NL, 1) && x_lines_compiled(p->n[0], p->m[0])) {
+          modes.push_back(5);
+          modes.push_back(-5);
+        }
         const int nm = (int)modes.size();
         for (int li = 0; li < nm * nm; ++li) {   // (forward, inverse) variants
           p->x_lpb = modes[li % nm];

@@ -9,6 +9,8 @@
 // and output are in natural order; the buffers alternate between stages.
 #pragma once
 
+#include <type_traits>
+
 #include "vie_internal.cuh"
 
 namespace vie {
@@ -34,10 +36,62 @@ template <typename V> struct real_of;
 template <> struct real_of<float2> { typedef float type; };
 template <> struct real_of<double2> { typedef double type; };
 
+// complex64 butterflies in packed FP32 instructions: sums and real scalings
+// of a complex value are one instruction, the rotations by i ride on
+// differences formed with their parts exchanged.  9 instead of 16
+// instructions at radix 4, 20 instead of 40 at radix 5.
+template <bool INV>
+__device__ __forceinline__ void dft_small_packed(float2* a, int r) {
+  constexpr float g = INV ? -1.f : 1.f;   // -i d = (d.y, -d.x) forward, +i d inverse
+  typedef RadixConst<float> C;
+  switch (r) {
+    case 2: {
+      const float2 b0 = add(a[0], a[1]), b1 = sub(a[0], a[1]);
+      a[0] = b0; a[1] = b1;
+      break;
+    }
+    case 3: {
+      const float2 s = add(a[1], a[2]), d = sub_swapped(a[1], a[2]);
+      const float2 m = fma2(s, -0.5f, a[0]);
+      a[0] = add(a[0], s);
+      a[1] = fma2(d, g * C::s3, -g * C::s3, m);
+      a[2] = fma2(d, -g * C::s3, g * C::s3, m);
+      break;
+    }
+    case 4: {
+      const float2 s02 = add(a[0], a[2]), d02 = sub(a[0], a[2]);
+      const float2 s13 = add(a[1], a[3]), d13 = sub_swapped(a[1], a[3]);
+      a[0] = add(s02, s13);
+      a[2] = sub(s02, s13);
+      a[1] = fma2(d13, g, -g, d02);
+      a[3] = fma2(d13, -g, g, d02);
+      break;
+    }
+    case 5: {
+      const float2 s14 = add(a[1], a[4]), d14 = sub_swapped(a[1], a[4]);
+      const float2 s23 = add(a[2], a[3]), d23 = sub_swapped(a[2], a[3]);
+      const float2 m1 = fma2(s14, C::c51, fma2(s23, C::c52, a[0]));
+      const float2 m2 = fma2(s14, C::c52, fma2(s23, C::c51, a[0]));
+      a[0] = add(a[0], add(s14, s23));
+      a[1] = fma2(d14, g * C::s51, -g * C::s51, fma2(d23, g * C::s52, -g * C::s52, m1));
+      a[4] = fma2(d14, -g * C::s51, g * C::s51, fma2(d23, -g * C::s52, g * C::s52, m1));
+      a[2] = fma2(d14, g * C::s52, -g * C::s52, fma2(d23, -g * C::s51, g * C::s51, m2));
+      a[3] = fma2(d14, -g * C::s52, g * C::s52, fma2(d23, g * C::s51, -g * C::s51, m2));
+      break;
+    }
+    default:
+      break;
+  }
+}
+
 // In-place r-point DFT of a[0..r); INV selects exp(+2 pi i tu / r).
 template <typename V, bool INV>
 __device__ __forceinline__ void dft_small(V* a, int r) {
   typedef typename real_of<V>::type R;
+  if constexpr (std::is_same<V, float2>::value) {
+    dft_small_packed<INV>(a, r);
+    return;
+  }
   switch (r) {
     case 2: {
       V b0 = add(a[0], a[1]), b1 = sub(a[0], a[1]);

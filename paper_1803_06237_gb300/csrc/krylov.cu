@@ -842,32 +842,13 @@ __device__ void coop_reduce(const ProbK* __restrict__ P, int count, const int* s
   }
 }
 
-// The FP64 least-squares step of problem q for column j by the block that
-// owns q.  The rotations of the cycle are kept multiplied out, Q = O_{j-1}
-// ... O_0 ((j + 1) x (j + 1), row-major, ld = m + 1 = ldh), so that applying
-// them to the new column is a matrix-vector product (a warp per row, lanes
-// over the columns, fixed-order reduction) instead of a chain of j
-// dependent rotations; thread 0 then forms the new rotation O_j on
-// (r_j, h_{j+1,j}), updates g and the status, and Q's rows j and j + 1 are
-// replaced by O_j applied to (row j, e_{j+1}).  sh: j + 2 double2.
-__device__ void coop_givens(const ProbK& q, int j, int ldh, double hn, double inv, double2* sh) {
-  double2* r = sh;
+// The end of the FP64 least-squares step of column j: thread 0 forms the new
+// rotation O_j on (r_j, h_{j+1,j} = hn), updates g and the status, and Q's
+// rows j and j + 1 are replaced by O_j applied to (row j, e_{j+1}).  r: the
+// column with the earlier rotations applied (shared memory, j + 2 entries).
+__device__ void lsq_column(const ProbK& q, int j, int ldh, double hn, double inv, double2* r) {
   __shared__ double2 rot[2];   // (c, 0), s
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int ldq = ldh;
-  __syncthreads();
-  for (int i = warp; i <= j; i += nw) {
-    double re = 0.0, im = 0.0;
-    for (int k = lane; k <= j; k += 32) {
-      const double2 g = j == 0 ? make_double2(1.0, 0.0) : q.Q[(size_t)i * ldq + k];
-      const double2 h = __ldcg(q.hcol + k);
-      re += g.x * h.x - g.y * h.y;
-      im += g.x * h.y + g.y * h.x;
-    }
-    re = warp_sum(re);
-    im = warp_sum(im);
-    if (lane == 0) r[i] = make_double2(re, im);
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
     SolveStatus* st = q.st;
@@ -933,6 +914,32 @@ __device__ void coop_givens(const ProbK& q, int j, int ldh, double hn, double in
         make_double2(-(s.x * gj.x + s.y * gj.y) + c * e.x, -(s.x * gj.y - s.y * gj.x) + c * e.y);
   }
   for (int i = threadIdx.x; i < j; i += blockDim.x) q.Q[(size_t)i * ldq + j + 1] = make_double2(0.0, 0.0);
+}
+
+// The FP64 least-squares step of problem q for column j by the block that
+// owns q.  The rotations of the cycle are kept multiplied out, Q = O_{j-1}
+// ... O_0 ((j + 1) x (j + 1), row-major, ld = m + 1 = ldh), so that applying
+// them to the new column is a matrix-vector product (a warp per row, lanes
+// over the columns, fixed-order reduction) instead of a chain of j
+// dependent rotations; lsq_column does the rest.  sh: j + 2 double2.
+__device__ void coop_givens(const ProbK& q, int j, int ldh, double hn, double inv, double2* sh) {
+  double2* r = sh;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int ldq = ldh;
+  __syncthreads();
+  for (int i = warp; i <= j; i += nw) {
+    double re = 0.0, im = 0.0;
+    for (int k = lane; k <= j; k += 32) {
+      const double2 g = j == 0 ? make_double2(1.0, 0.0) : q.Q[(size_t)i * ldq + k];
+      const double2 h = __ldcg(q.hcol + k);
+      re += g.x * h.x - g.y * h.y;
+      im += g.x * h.y + g.y * h.x;
+    }
+    re = warp_sum(re);
+    im = warp_sum(im);
+    if (lane == 0) r[i] = make_double2(re, im);
+  }
+  lsq_column(q, j, ldh, hn, inv, r);
 }
 
 // Step j (nv = j + 1 basis vectors) for the count problems of P after the
@@ -1049,6 +1056,300 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
         atomicExch(bar + 3, 0u);
       }
     }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The Gram-Schmidt step of one complex64 problem with w in registers
+// ---------------------------------------------------------------------------
+// Bound by reading the basis (j + 1 vectors, mostly from L2) once for the
+// products and once for the update of each pass.  What the step above spends
+// beside that goes: every thread of a worker block keeps its E elements of w
+// in registers from the first product to v_{j+1}, so w is read once and never
+// written; every block sums the partials of all blocks by itself (the sums
+// are identical, in a fixed order), so a pass has two grid barriers instead
+// of three or four; and the last block owns no elements: it sums the same
+// partials and does the FP64 least-squares step while the workers update w
+// and write v_{j+1}.  600 x 23 x 11, restart 30: 60 us a step against 103
+// with the step above (operator excluded).
+//
+// Barrier: a counter that only grows.  A block's ticket t belongs to barrier
+// t / nblocks, which is complete when the counter reaches the next multiple
+// of nblocks.  The wait is bounded by the abort word as in grid_barrier.
+__device__ __forceinline__ bool ticket_barrier(unsigned* bar, unsigned nblocks) {
+  __shared__ int ok_s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned t = atomicAdd(bar, 1u);
+    const unsigned target = (t / nblocks + 1u) * nblocks;
+    int ok = 1;
+    unsigned seen;
+    const long long t0 = clock64();
+    while (true) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      if ((int)(seen - target) >= 0) break;
+      if (clock64() - t0 > kBarrierCycles) {
+        atomicExch(bar + 2, 1u);
+        ok = 0;
+        break;
+      }
+    }
+    ok_s = ok && *(volatile unsigned*)(bar + 2) == 0u;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
+constexpr int kStepThreads = 512;
+constexpr int kStepWarps = kStepThreads / 32;
+constexpr int kDotGroup = 16;   // vectors whose products a thread accumulates at a time
+
+// Sum over a warp of 32 values per lane: lane l ends with value l (31
+// shuffles instead of 5 per value).
+__device__ __forceinline__ float warp_transpose_sum(float (&a)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const float keep = up ? a[k + o] : a[k], give = up ? a[k] : a[k + o];
+      a[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  return a[0];
+}
+
+// vectors loaded together: about 24 loads in flight a thread
+template <int E> __host__ __device__ constexpr int step_vectors() { return E <= 2 ? 8 : E <= 6 ? 4 : E <= 8 ? 2 : 1; }
+
+// Block partials of conj(V_i) w, i < nv -> partial[i nblk + blockIdx.x].
+template <int E>
+__device__ void step_dots(const float2* __restrict__ V, size_t n, int nv, size_t k0, int own, const float2 (&w)[E],
+                          double2* __restrict__ partial, int nblk, float (*red)[kStepWarps][32]) {
+  constexpr int G = step_vectors<E>();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i0 = 0; i0 < nv; i0 += kDotGroup) {
+    float acc[2 * kDotGroup];
+#pragma unroll
+    for (int u = 0; u < 2 * kDotGroup; ++u) acc[u] = 0.f;
+#pragma unroll
+    for (int g = 0; g < kDotGroup; g += G) {
+      if (i0 + g < nv) {
+        float2 a[G][E];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          const float2* v = V + (size_t)min(i0 + g + u, nv - 1) * n + k0;
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const int k = threadIdx.x + e * kStepThreads;
+            a[u][e] = k < own ? v[k] : make_float2(0.f, 0.f);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            acc[2 * (g + u)] += a[u][e].x * w[e].x + a[u][e].y * w[e].y;
+            acc[2 * (g + u) + 1] += a[u][e].x * w[e].y - a[u][e].y * w[e].x;
+          }
+      }
+    }
+    red[0][warp][lane] = warp_transpose_sum(acc);
+    __syncthreads();
+    if (threadIdx.x < 32 && i0 + (threadIdx.x >> 1) < nv) {
+      double t = 0.0;
+#pragma unroll
+      for (int k = 0; k < kStepWarps; ++k) t += (double)red[0][k][threadIdx.x];
+      ((double*)(partial + (size_t)(i0 + (threadIdx.x >> 1)) * nblk + blockIdx.x))[threadIdx.x & 1] = t;
+    }
+    __syncthreads();
+  }
+}
+
+// w -= V h, h in shared memory
+template <int E>
+__device__ void step_update(const float2* __restrict__ V, size_t n, int nv, size_t k0, int own, float2 (&w)[E],
+                            const float2* h) {
+  constexpr int G = step_vectors<E>();
+  for (int i0 = 0; i0 < nv; i0 += G) {
+    float2 a[G][E];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const float2* v = V + (size_t)min(i0 + u, nv - 1) * n + k0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int k = threadIdx.x + e * kStepThreads;
+        a[u][e] = k < own ? v[k] : make_float2(0.f, 0.f);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const float2 hu = i0 + u < nv ? h[i0 + u] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        w[e].x -= a[u][e].x * hu.x - a[u][e].y * hu.y;
+        w[e].y -= a[u][e].x * hu.y + a[u][e].y * hu.x;
+      }
+    }
+  }
+}
+
+// block partial of |w|^2 -> *out
+template <int E>
+__device__ void step_norm(const float2 (&w)[E], double2* out, float (*red)[kStepWarps][32]) {
+  float t = 0.f;
+#pragma unroll
+  for (int e = 0; e < E; ++e) t += w[e].x * w[e].x + w[e].y * w[e].y;
+  t = warp_sum(t);
+  if ((threadIdx.x & 31) == 0) red[0][0][threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double u = 0.0;
+    for (int k = 0; k < kStepWarps; ++k) u += (double)red[0][0][k];
+    *out = make_double2(u, 0.0);
+  }
+}
+
+// coefficients of every vector: the sum of its partials, one warp per vector
+__device__ void step_coefficients(const double2* __restrict__ partial, int nv, int workers, int nblk,
+                                  double2* __restrict__ hd, float2* __restrict__ hf) {
+  for (int i = threadIdx.x >> 5; i < nv; i += kStepWarps) {
+    const double2 t = warp_sum_partials(partial + (size_t)i * nblk, workers);
+    if ((threadIdx.x & 31) == 0) {
+      hd[i] = t;
+      hf[i] = make_float2((float)t.x, (float)t.y);
+    }
+  }
+  __syncthreads();
+}
+
+// r += Q h for the least-squares step (Q: the product of the cycle's
+// rotations, the identity for the first column): warp per row
+__device__ void step_rotate(const ProbK& q, int j, int ldq, const double2* __restrict__ h, double2* __restrict__ r,
+                            bool first) {
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i <= j; i += kStepWarps) {
+    double re = 0.0, im = 0.0;
+    for (int k = lane; k <= j; k += 32) {
+      const double2 g = j == 0 ? make_double2(1.0, 0.0) : q.Q[(size_t)i * ldq + k];
+      re += g.x * h[k].x - g.y * h[k].y;
+      im += g.x * h[k].y + g.y * h[k].x;
+    }
+    re = warp_sum(re);
+    im = warp_sum(im);
+    if (lane == 0) r[i] = first ? make_double2(re, im) : make_double2(r[i].x + re, r[i].y + im);
+  }
+  __syncthreads();
+}
+
+// Step j = nv - 1 of problem P[0]; worker blocks 0 .. gridDim.x - 2 own
+// `chunk` elements each.  Dynamic shared memory: nv double2 (coefficients),
+// nv + 1 double2 (the rotated column), nv float2.
+template <int E>
+__global__ void __launch_bounds__(kStepThreads, 1) arnoldi_step1_kernel(const ProbK* __restrict__ P, int nv, int ldh,
+                                                                        int chunk, unsigned* bar,
+                                                                        cudaGraphConditionalHandle next,
+                                                                        int set_next) {
+  const ProbK& q = P[0];
+  if (!q.st->active) return;   // written only by the last block, after a barrier every block has passed
+  extern __shared__ double2 step_raw[];
+  __shared__ float red[1][kStepWarps][32];
+  __shared__ double norm_s;
+  double2* hd = step_raw;
+  double2* r = hd + nv;
+  float2* hf = reinterpret_cast<float2*>(r + nv + 1);
+  const int j = nv - 1, nblk = gridDim.x, workers = nblk - 1;
+  const bool owner = (int)blockIdx.x == workers;
+  const size_t n = q.n, k0 = (size_t)blockIdx.x * chunk;
+  const int own = owner || k0 >= n ? 0 : (int)min((size_t)chunk, n - k0);
+  const float2* __restrict__ V = (const float2*)q.V;
+  float2 w[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int k = threadIdx.x + e * kStepThreads;
+    w[e] = k < own ? ((const float2*)q.w)[k0 + k] : make_float2(0.f, 0.f);
+  }
+  if (!owner) step_dots<E>(V, n, nv, k0, own, w, q.partial, nblk, red);
+  if (!ticket_barrier(bar, nblk)) return;
+  step_coefficients(q.partial, nv, workers, nblk, hd, hf);
+  if (!owner) {
+    step_update<E>(V, n, nv, k0, own, w, hf);
+    step_norm<E>(w, q.partial + (size_t)nv * nblk + blockIdx.x, red);
+  } else {
+    step_rotate(q, j, ldh, hd, r, true);
+  }
+  if (!ticket_barrier(bar, nblk)) return;
+  // ||w'|| and the second-pass decision, identical in every block:
+  // ||w'||^2 < (||w'||^2 + ||h1||^2) / 2
+  if (threadIdx.x < 32) {
+    const double t = warp_sum_partials(q.partial + (size_t)nv * nblk, workers).x;
+    double h2 = 0.0;
+    for (int i = threadIdx.x; i < nv; i += 32) h2 += hd[i].x * hd[i].x + hd[i].y * hd[i].y;
+    h2 = warp_sum(h2);
+    if (threadIdx.x == 0) norm_s = t < 0.5 * (t + h2) ? -1.0 : t;
+  }
+  __syncthreads();
+  const bool again = norm_s < 0.0;
+  if (again) {
+    if (!owner) step_dots<E>(V, n, nv, k0, own, w, q.partial, nblk, red);
+    if (!ticket_barrier(bar, nblk)) return;
+    step_coefficients(q.partial, nv, workers, nblk, hd, hf);
+    if (!owner) {
+      step_update<E>(V, n, nv, k0, own, w, hf);
+      step_norm<E>(w, q.partial + (size_t)(nv + 1) * nblk + blockIdx.x, red);
+    } else {
+      step_rotate(q, j, ldh, hd, r, false);
+    }
+    if (!ticket_barrier(bar, nblk)) return;
+    if (threadIdx.x < 32) {
+      const double t = warp_sum_partials(q.partial + (size_t)(nv + 1) * nblk, workers).x;
+      if (threadIdx.x == 0) norm_s = t;
+    }
+    __syncthreads();
+  }
+  const double hn = sqrt(norm_s);
+  const double inv = (hn > 0.0 && isfinite(hn)) ? 1.0 / hn : 0.0;
+  if (!owner) {
+    const float sc = (float)inv;
+    float2* __restrict__ v = (float2*)q.V + (size_t)nv * n + k0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int k = threadIdx.x + e * kStepThreads;
+      if (k < own) v[k] = make_float2(w[e].x * sc, w[e].y * sc);
+    }
+    return;
+  }
+  if (threadIdx.x == 0) {
+    q.st->reorth = again;
+    q.st->reorth_count += again;
+  }
+  lsq_column(q, j, ldh, hn, inv, r);
+  if (set_next && threadIdx.x == 0) cudaGraphSetConditional(next, q.st->active ? 1u : 0u);
+}
+
+// E elements a thread for n elements over `workers` blocks; 0: too many
+static int step_elements(size_t n, int workers) {
+  const size_t per = (n + workers - 1) / workers, e = (per + kStepThreads - 1) / kStepThreads;
+  for (int k : {2, 4, 6, 8, 12, 16})
+    if (e <= (size_t)k) return k;
+  return 0;
+}
+
+static size_t step_smem(int nv) { return (size_t)(2 * nv + 1) * sizeof(double2) + (size_t)nv * sizeof(float2); }
+
+// the kernel for a problem, or null
+typedef void (*StepKernel)(const ProbK*, int, int, int, unsigned*, cudaGraphConditionalHandle, int);
+static StepKernel step_kernel(int e) {
+  switch (e) {
+    case 2: return arnoldi_step1_kernel<2>;
+    case 4: return arnoldi_step1_kernel<4>;
+    case 6: return arnoldi_step1_kernel<6>;
+    case 8: return arnoldi_step1_kernel<8>;
+    case 12: return arnoldi_step1_kernel<12>;
+    case 16: return arnoldi_step1_kernel<16>;
+    default: return nullptr;
   }
 }
 
@@ -1293,6 +1594,8 @@ struct BatchCall {
   unsigned* bar = nullptr;          // grid barrier of the cooperative step (arrivals, generation, abort)
   unsigned* bar_host = nullptr;     // pinned copy of the abort word
   int coop_blocks = 0;              // blocks of the cooperative step (0: separate kernels)
+  int step_e = 0;                   // elements a thread of the one-problem step (0: not used)
+  int step_blocks = 0;              //   and its blocks
   bool resident = false;            // the whole solve runs as one graph launch
   ResState* rs = nullptr;           // device, one per problem (resident solve)
   ResCtl* ctl = nullptr;            // device (resident solve)
@@ -1326,6 +1629,31 @@ static int coop_blocks_for(int m) {
   }
   int nb = sms * (per > 1 ? 1 : per);
   return nb > kDotBlocks ? kDotBlocks : nb;
+}
+
+// One complex64 problem: blocks and elements a thread of the one-problem
+// step, or zeros where it does not apply (more elements than 16 a thread, no
+// cooperative launch).  Small problems take fewer blocks: a barrier costs
+// less than the elements it would spread.
+static void step_shape(size_t n, int m, int* blocks, int* e) {
+  *blocks = *e = 0;
+  int dev = 0, coop = 0, sms = 0, per = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (!coop || sms < 2) return;
+  int nb = sms < kDotBlocks ? sms : kDotBlocks;
+  const size_t want = (n + 2 * kStepThreads - 1) / (2 * kStepThreads) + 1;
+  if ((size_t)nb > want) nb = (int)want;
+  const int k = step_elements(n, nb - 1);
+  if (!k || step_smem(m) > 48 * 1024 ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel(k), kStepThreads, step_smem(m)) != cudaSuccess ||
+      per < 1) {
+    cudaGetLastError();
+    return;
+  }
+  *blocks = nb;
+  *e = k;
 }
 
 static vie_status upload_list(BatchCall& c, const std::vector<int>& list, cudaStream_t s) {
@@ -1450,6 +1778,24 @@ static vie_status enqueue_step(BatchCall& c, const std::vector<int>& list, const
   vie_status ms = apply_list(c, live, dtype, APPLY_Z, j, flexible, s);
   if (ms != VIE_OK) return ms;
   const int nv = j + 1;
+  if (sizeof(V) == sizeof(float2) && c.step_e) {
+    const size_t n = c.host[list[0]].n;
+    const int workers = c.step_blocks - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)c.step_blocks);
+    cfg.blockDim = dim3(kStepThreads);
+    cfg.dynamicSmemBytes = step_smem(nv);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    VIE_CUDA_TRY(cudaLaunchKernelEx(&cfg, step_kernel(c.step_e), (const ProbK*)c.table, nv, m + 1,
+                                    (int)((n + workers - 1) / workers), c.bar, next, next_set ? 1 : 0));
+    if (next_set) *next_set = true;
+    return VIE_OK;
+  }
   if (c.coop_blocks > 0 && P <= (unsigned)kCoopMaxProblems) {
     // the whole Gram-Schmidt step, ||w||, v_{j+1} and the Givens step in one
     // cooperative launch
@@ -1496,9 +1842,11 @@ __global__ void next_step_condition_kernel(const ProbK* __restrict__ P, int coun
   cudaGraphSetConditional(h, any ? 1u : 0u);
 }
 
-// A whole GMRES cycle as one CUDA graph: the start vector, then one
-// conditional (IF) node per Arnoldi step whose body ends by setting the next
-// step's condition from the problems' device status, then the back
+constexpr int kStepsPerNode = 6;
+
+// A whole GMRES cycle as one CUDA graph: the start vector, then conditional
+// (IF) nodes of a few Arnoldi steps whose bodies end by setting the next
+// node's condition from the problems' device status, then the back
 // substitution and the update of x.  Launched once per cycle, it runs every
 // step on the device with no host round trip; the steps after the last
 // active problem stopped are skipped by the device.  The instantiated graph
@@ -1529,15 +1877,21 @@ static vie_status build_cycle_graph(BatchCall& c, CycleGraph& G, const std::vect
   if (!G.cap) VIE_CUDA_TRY(cudaStreamCreateWithFlags(&G.cap, cudaStreamNonBlocking));
   const unsigned P = (unsigned)list.size();
   VIE_CUDA_TRY(cudaGraphCreate(&G.graph, 0));
-  // handles: [0] start (always), [1 + j] step j (step 0 always, later steps
-  // set by the step before), [jmax + 1] finish (always)
-  std::vector<cudaGraphConditionalHandle> h(jmax + 2);
-  for (int k = 0; k < jmax + 2; ++k) {
-    const unsigned def = (k == 0 || k == 1 || k == jmax + 1) ? 1u : 0u;
+  // One IF node per kStepsPerNode steps: handles [0] start (always), [1 + b]
+  // the b-th block of steps (the first always, later ones set by the last
+  // step of the block before), then finish (always).  Entering a node costs
+  // about 10 us; a step of a problem that has stopped returns at once from
+  // every launch.  Preconditioned steps and the JM-VIE, whose operators do not
+  // skip, keep one step per node.
+  const int per = flexible || c.jm ? 1 : kStepsPerNode;
+  const int nodes = (jmax + per - 1) / per + 2;
+  std::vector<cudaGraphConditionalHandle> h(nodes);
+  for (int k = 0; k < nodes; ++k) {
+    const unsigned def = (k == 0 || k == 1 || k == nodes - 1) ? 1u : 0u;
     VIE_CUDA_TRY(cudaGraphConditionalHandleCreate(&h[k], G.graph, def, cudaGraphCondAssignDefault));
   }
   cudaGraphNode_t prev = nullptr;
-  for (int k = 0; k < jmax + 2; ++k) {
+  for (int k = 0; k < nodes; ++k) {
     cudaGraphNodeParams cp = {};
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.handle = h[k];
@@ -1550,12 +1904,16 @@ static vie_status build_cycle_graph(BatchCall& c, CycleGraph& G, const std::vect
     vie_status st = VIE_OK;
     if (k == 0) {
       start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, G.cap>>>(c.table);
-    } else if (k <= jmax) {
-      bool set = false;
-      st = enqueue_step<V>(c, list, list, k - 1, m, dtype, flexible, precond, precond_ctx, gx, G.cap,
-                           k < jmax ? h[k + 1] : 0, k < jmax ? &set : nullptr);
-      if (st == VIE_OK && k < jmax && !set)
-        next_step_condition_kernel<<<1, 32, 0, G.cap>>>(c.table, (int)P, h[k + 1]);
+    } else if (k < nodes - 1) {
+      const int j0 = (k - 1) * per, j1 = j0 + per < jmax ? j0 + per : jmax;
+      for (int j = j0; j < j1 && st == VIE_OK; ++j) {
+        const bool sets = j == j1 - 1 && j1 < jmax;   // the block's last step, another block follows
+        bool set = false;
+        st = enqueue_step<V>(c, list, list, j, m, dtype, flexible, precond, precond_ctx, gx, G.cap,
+                             sets ? h[k + 1] : 0, sets ? &set : nullptr);
+        if (st == VIE_OK && sets && !set)
+          next_step_condition_kernel<<<1, 32, 0, G.cap>>>(c.table, (int)P, h[k + 1]);
+      }
     } else {
       backsolve_kernel<<<P, kThreads, 0, G.cap>>>(c.table, m + 1);
       update_x_kernel<V><<<dim3(gx, P), kThreads, (size_t)m * sizeof(typename Acc<V>::T), G.cap>>>(c.table);
@@ -1916,6 +2274,8 @@ vie_status solve_batch_impl(vie_plan* const* plans, int count, const double2* co
   c.coop_blocks = (count <= kCoopMaxProblems)
                       ? (dtype == VIE_C64 ? coop_blocks_for<float2>(m) : coop_blocks_for<double2>(m))
                       : 0;
+  if (count == 1 && dtype == VIE_C64)
+    step_shape((size_t)(jm ? 6 : 3) * plans[0]->n[0] * plans[0]->n[1] * plans[0]->n[2], m, &c.step_blocks, &c.step_e);
   for (int i = 0; i < count; ++i) {
     KrylovWork* k = nullptr;
     vie_status st = ensure_work(plans[i], m, dtype, flexible, &k, jm ? 6 : 3);

@@ -25,36 +25,11 @@
 #include <string.h>
 
 #include "fft.cuh"
+#include "passes.cuh"
 #include "regfft.cuh"
 #include "vie_internal.cuh"
 
 namespace vie {
-
-template <typename V> __device__ __forceinline__ V zero_c();
-template <> __device__ __forceinline__ float2 zero_c<float2>() { return make_float2(0.f, 0.f); }
-template <> __device__ __forceinline__ double2 zero_c<double2>() { return make_double2(0.0, 0.0); }
-
-// Per-problem pointers of one launch: blockIdx.y selects the problem.  All
-// problems of a launch share the grid and circulant sizes (and twiddles).
-constexpr int kMaxBatch = 16;
-template <typename V>
-struct PassPtrs {
-  const V* x[kMaxBatch];
-  V* y[kMaxBatch];
-  V* work[kMaxBatch];
-  const V* ghat[kMaxBatch];
-  const V* M[kMaxBatch];
-  V* work2[kMaxBatch];        // y-pass buffer of the split pass B (or null)
-  const int* live[kMaxBatch]; // per problem: null, or a device flag; 0 skips the problem (its blocks return)
-};
-
-// A problem whose live flag is 0 is skipped by every block of every pass
-// (blockIdx.y is the problem in all grouped launches).
-template <typename V>
-__device__ __forceinline__ bool skip_problem(const PassPtrs<V>& pp) {
-  const int* f = pp.live[blockIdx.y];
-  return f != nullptr && *(const volatile int*)f == 0;
-}
 
 // ---------------------------------------------------------------------------
 // pass A
@@ -93,10 +68,6 @@ __global__ void __launch_bounds__(256) pass_a_kernel(const __grid_constant__ Pas
 // ---------------------------------------------------------------------------
 // pass B
 // ---------------------------------------------------------------------------
-struct PassBGeom {
-  int ny, nz, NL, Mx, My, Mz, Ky, Kz;
-};
-
 template <typename V>
 __global__ void __launch_bounds__(256) pass_b_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g,
                                                      Radices ry, Radices rz, const V* __restrict__ twyg,
@@ -1142,167 +1113,63 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
   }
 }
 
-// Mx = L1 L2 L3 factorisations with a three-factor register x pass, and the
-// compiled line lengths.
-#define VIE_PASS_X3_SIZES(X) X(10, 12, 10)
-#define VIE_PASS_X3_FIXED(X) X(10, 12, 10, 600)
+// The two kernels above are compiled for the benchmark guide's lines: complex64,
+// 600 values into 1200, five lines per block (x_lines_five).  There they take
+// 9 and 11 us where the passes with run-time radices (any_x.cuh) take 10 and
+// 13; at every other size those are the faster ones.
+template <typename V, typename Kernel, typename... Args>
+static vie_status launch_x_lines(Kernel kernel, dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args) {
+  VIE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VIE_CUDA_TRY(launch_pdl(kernel, blocks, dim3(threads), smem, s, args...));
+  return VIE_OK;
+}
 
-template <typename V, int L1, int L2, int L3, int LPB, int NX>
-static vie_status launch_x3_lpb(bool forward, const PassPtrs<V>& pp, int count, int nx, int nyz, int NL,
-                                const V* twx, int mode, cudaStream_t s, bool* done, int gsz) {
-  typedef X3<L1, L2, L3> G;
-  constexpr int R1 = pitch_mod16(G::T1 * LPB, LPB);
-  constexpr int R2 = pitch_mod16(L1 * LPB, LPB);
-  const int P = pitch_mod16(nx, LPB);
-  const bool operands = !forward && mode != MODE_PLAIN;
-  const size_t smem = (size_t)(G::MX + L1 + L2 + L3 + L3 * R1 + G::M * R2 + LPB * P +
-                               (forward ? 0 : (operands ? 2 * LPB * nx : 0))) * sizeof(V);
-  if (smem > 200 * 1024) { *done = false; return VIE_OK; }
+bool x_lines_compiled(int nx, int Mx) { return nx == 600 && Mx == 1200; }
+
+// lpb -5: three-factor kernel, 5: four-step kernel
+static vie_status launch_x_five(bool forward, int lpb, const PassPtrs<float2>& pp, int count, int nx, int nyz, int NL,
+                                const float2* twx, int mode, cudaStream_t s, int gsz) {
+  constexpr int LPB = 5;
   const dim3 blocks((unsigned)((NL + LPB - 1) / LPB), (unsigned)count);
-  const dim3 threads(LPB * G::NT);
-  if (forward) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a3_kernel<V, L1, L2, L3, LPB, NX>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    VIE_CUDA_TRY(launch_pdl(pass_a3_kernel<V, L1, L2, L3, LPB, NX>, blocks, threads, smem, s, pp, nx, NL, twx, gsz));
-  } else {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c3_kernel<V, L1, L2, L3, LPB, NX>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    VIE_CUDA_TRY(launch_pdl(pass_c3_kernel<V, L1, L2, L3, LPB, NX>, blocks, threads, smem, s, pp, nx, nyz, NL, twx,
-                            mode, gsz));
+  const int P = pitch_mod16(nx, LPB);
+  const size_t operands = forward ? 0 : 2 * LPB * nx;   // epilogue rows of x and M
+  if (lpb < 0) {
+    typedef X3<10, 12, 10> G;
+    constexpr int R1 = pitch_mod16(G::T1 * LPB, LPB), R2 = pitch_mod16(10 * LPB, LPB);
+    const size_t smem = (size_t)(G::MX + 10 + 12 + 10 + 10 * R1 + G::M * R2 + LPB * P + operands) * sizeof(float2);
+    if (forward)
+      return launch_x_lines<float2>(pass_a3_kernel<float2, 10, 12, 10, LPB, 600>, blocks, LPB * G::NT, smem, s, pp, nx,
+                                    NL, twx, gsz);
+    return launch_x_lines<float2>(pass_c3_kernel<float2, 10, 12, 10, LPB, 600>, blocks, LPB * G::NT, smem, s, pp, nx,
+                                  nyz, NL, twx, mode, gsz);
   }
-  VIE_LAUNCH_CHECK();
-  *done = true;
-  return VIE_OK;
+  constexpr int R = pitch_mod16(40 * LPB, LPB);
+  const size_t smem = (size_t)(1200 + 40 + 30 + 30 * R + LPB * P + operands) * sizeof(float2);
+  if (forward)
+    return launch_x_lines<float2>(pass_a4_kernel<float2, 40, 30, LPB, 600>, blocks, LPB * 40, smem, s, pp, nx, NL, twx,
+                                  gsz);
+  return launch_x_lines<float2>(pass_c4_kernel<float2, 40, 30, LPB, 600>, blocks, LPB * 40, smem, s, pp, nx, nyz, NL,
+                                twx, mode, gsz);
 }
 
-// lpb: 1, 2 or 5 lines per block (0: 5 where x_lines_five holds and the
-// complex64 kernel with the line length compiled in exists, else 2)
-template <typename V, int L1, int L2, int L3, int NX = 0>
-static vie_status launch_x3(bool forward, const PassPtrs<V>& pp, int count, int nx, int nyz, int NL, const V* twx,
-                            int mode, cudaStream_t s, bool* done, int lpb, int gsz) {
-  if (lpb == 1) return launch_x3_lpb<V, L1, L2, L3, 1, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-  if constexpr (sizeof(V) == sizeof(float2) && NX > 0) {
-    if (lpb == 5 || (lpb == 0 && x_lines_five(NL, count)))
-      return launch_x3_lpb<V, L1, L2, L3, 5, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-  }
-  return launch_x3_lpb<V, L1, L2, L3, 2, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-}
-
-// factors (L1, L2, L3) of Mx with a compiled three-factor kernel, or (0, 0, 0)
-void x3_factors(int mx, int* l1, int* l2, int* l3) {
-  *l1 = *l2 = *l3 = 0;
-#define VIE_X(a, b, c) if (mx == a * b * c && *l1 == 0) { *l1 = a; *l2 = b; *l3 = c; }
-  VIE_PASS_X3_SIZES(VIE_X)
-#undef VIE_X
-}
+// An x pass of a plan: the compiled five-line kernels where they apply (or the
+// tuner chose them: lpb), else the run-time radices, else the generic kernel.
+template <typename V>
+static vie_status launch_x_generic(bool forward, const PassPtrs<V>& pp, int count, int n, int nyz, int NL,
+                                   const Radices& rd, const V* tw, int mode, cudaStream_t s, int gsz);
 
 template <typename V>
-static vie_status dispatch_x3(bool forward, int l1, int l2, int l3, const PassPtrs<V>& pp, int count, int nx,
-                              int nyz, int NL, const V* twx, int mode, cudaStream_t s, bool* done, int lpb,
-                              int gsz) {
-  *done = false;
-#define VIE_Y(a, b, c, d)                                        \
-  if (l1 == a && l2 == b && l3 == c && nx == d)                   \
-    return launch_x3<V, a, b, c, d>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, lpb, gsz);
-  VIE_PASS_X3_FIXED(VIE_Y)
-#undef VIE_Y
-#define VIE_X(a, b, c) \
-  if (l1 == a && l2 == b && l3 == c) return launch_x3<V, a, b, c>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, lpb, gsz);
-  VIE_PASS_X3_SIZES(VIE_X)
-#undef VIE_X
-  return VIE_OK;
-}
-
-// Mx = L1 x L2 factorisations with a four-step register x pass.
-#define VIE_PASS_X4_SIZES(X) \
-  X(40, 30) X(24, 25) X(24, 30) X(30, 30) X(45, 25) X(45, 30) X(50, 30) X(40, 40) X(20, 20)
-// (L1, L2, NX) with the line length compiled in: 600 values (12 um at 20 nm
-// along x; the ring resonator's 600 y-voxels) into 1200 = 40 x 30.
-#define VIE_PASS_X4_FIXED(X) X(40, 30, 600)
-
-template <typename V, int L1, int L2, int LPB, int NX>
-static vie_status launch_x4_lpb(bool forward, const PassPtrs<V>& pp, int count, int nx, int nyz, int NL,
-                                const V* twx, int mode, cudaStream_t s, bool* done, int gsz) {
-  {
-    constexpr int R = pitch_mod16(L1 * LPB, LPB);
-    constexpr int NT = LPB * (L1 > L2 ? L1 : L2);
-    const int P = pitch_mod16(nx, LPB);
-    const bool operands = !forward && mode != MODE_PLAIN;   // epilogue rows of x and M
-    const size_t smem = (size_t)(L1 * L2 + L1 + L2 + L2 * R + LPB * P + (operands ? 2 * LPB * nx : 0)) * sizeof(V);
-    if (smem > 200 * 1024) { *done = false; return VIE_OK; }
-    const dim3 blocks((unsigned)((NL + LPB - 1) / LPB), (unsigned)count);
-    if (forward) {
-      VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a4_kernel<V, L1, L2, LPB, NX>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      VIE_CUDA_TRY(launch_pdl(pass_a4_kernel<V, L1, L2, LPB, NX>, blocks, dim3(NT), smem, s, pp, nx, NL, twx, gsz));
-    } else {
-      VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c4_kernel<V, L1, L2, LPB, NX>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      VIE_CUDA_TRY(
-          launch_pdl(pass_c4_kernel<V, L1, L2, LPB, NX>, blocks, dim3(NT), smem, s, pp, nx, nyz, NL, twx, mode, gsz));
-    }
-    VIE_LAUNCH_CHECK();
-    *done = true;
-    return VIE_OK;
+static vie_status launch_x(bool forward, int lpb, const AxisPlan& ax, const PassPtrs<V>& pp, int count, int n, int nyz,
+                           int NL, const V* tw, int mode, cudaStream_t s, int gsz) {
+  if constexpr (sizeof(V) == sizeof(float2)) {
+    const int choice = lpb ? lpb : forward ? -5 : 5;
+    if (x_lines_five(NL, count) && x_lines_compiled(n, ax.len) && mode != MODE_PLAIN)
+      return launch_x_five(forward, choice, pp, count, n, nyz, NL, tw, mode, s, gsz);
   }
-}
-
-// Four lines per block, or two when four would leave fewer than one block
-// per SM (more blocks hide the latency of the small per-line work), unless
-// the plan's tuner chose (lpb = 2 or 4).  Inverse passes with at least four
-// blocks of eight lines per SM (complex64) take eight lines when they fit:
-// each transposed row read is then 64 contiguous bytes, which matters once
-// the workspace no longer fits in L2 (forward passes measured slower so).
-template <typename V, int L1, int L2, int NX = 0>
-static vie_status launch_x4(bool forward, const PassPtrs<V>& pp, int count, int nx, int nyz, int NL,
-                            const V* twx, int mode, cudaStream_t s, bool* done, int lpb, int gsz) {
-  if constexpr (sizeof(V) == sizeof(float2) || (L1 <= 30 && L2 <= 30)) {
-    if constexpr (sizeof(V) == sizeof(float2)) {
-      const long blocks8 = (long)((NL + 7) / 8) * count;
-      if (lpb == 8 || (lpb == 0 && !forward && blocks8 >= 4L * kSMs)) {
-        vie_status st = launch_x4_lpb<V, L1, L2, 8, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-        if (st != VIE_OK || *done) return st;
-      }
-    }
-    if constexpr (sizeof(V) == sizeof(float2) && NX > 0) {
-      if (lpb == 5 || (lpb == 0 && x_lines_five(NL, count)))
-        return launch_x4_lpb<V, L1, L2, 5, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-    }
-    const long blocks4 = (long)((NL + 3) / 4) * count;
-    if (lpb == 2) return launch_x4_lpb<V, L1, L2, 2, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-    if (lpb == 4) return launch_x4_lpb<V, L1, L2, 4, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-    if (blocks4 < kSMs)
-      return launch_x4_lpb<V, L1, L2, 2, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-    return launch_x4_lpb<V, L1, L2, 4, NX>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, gsz);
-  } else {
-    *done = false;
-    return VIE_OK;
-  }
-}
-
-// factor (L1, L2) of Mx with a compiled four-step kernel, or (0, 0)
-void x4_factors(int mx, int* l1, int* l2) {
-  *l1 = 0;
-  *l2 = 0;
-#define VIE_X(a, b) if (mx == a * b && *l1 == 0) { *l1 = a; *l2 = b; }
-  VIE_PASS_X4_SIZES(VIE_X)
-#undef VIE_X
-}
-
-template <typename V>
-static vie_status dispatch_x4(bool forward, int l1, int l2, const PassPtrs<V>& pp, int count, int nx, int nyz,
-                              int NL, const V* twx, int mode, cudaStream_t s, bool* done, int lpb, int gsz) {
-  *done = false;
-#define VIE_X(a, b) \
-  if (l1 == a && l2 == b) return launch_x4<V, a, b>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, lpb, gsz);
-#define VIE_Y(a, b, c)                      \
-  if (l1 == a && l2 == b && nx == c)          \
-    return launch_x4<V, a, b, c>(forward, pp, count, nx, nyz, NL, twx, mode, s, done, lpb, gsz);
-  VIE_PASS_X4_FIXED(VIE_Y)
-#undef VIE_Y
-  VIE_PASS_X4_SIZES(VIE_X)
-#undef VIE_X
-  return VIE_OK;
+  bool done = false;
+  vie_status st = launch_x_any<V>(forward, pp, count, n, nyz, NL, ax.len, tw, mode, s, gsz, &done);
+  if (st != VIE_OK || done) return st;
+  return launch_x_generic<V>(forward, pp, count, n, nyz, NL, radices_of(ax), tw, mode, s, gsz);
 }
 
 // ---------------------------------------------------------------------------
@@ -1351,8 +1218,6 @@ template <typename V>
 static vie_status run_split_b(const vie_plan* p, const PassPtrs<V>& pp, int count, const PassBGeom& g,
                               const V* twy, const V* twz, cudaStream_t s) {
   const int NLy = g.Mx * 3 * g.nz;
-  int l1 = 0, l2 = 0;
-  x4_factors(g.My, &l1, &l2);
   PassPtrs<V> p1 = pp;   // B1: lines of the slab -> Y
   PassPtrs<V> p3 = pp;   // B3: Y -> lines of the slab
   for (int k = 0; k < count; ++k) {
@@ -1361,18 +1226,10 @@ static vie_status run_split_b(const vie_plan* p, const PassPtrs<V>& pp, int coun
     p3.work[k] = pp.work2[k];
     p3.y[k] = pp.work[k];
   }
-  bool done = false;
-  vie_status st = VIE_OK;
   const int gsz = 3 * g.nz;   // one group of lines per kx: Y[kx][ky][l]
-  if (l1) st = dispatch_x4<V>(true, l1, l2, p1, count, g.ny, 1, NLy, twy, MODE_PLAIN, s, &done, 0, gsz);
-  if (st == VIE_OK && !done)
-    st = launch_x_generic<V>(true, p1, count, g.ny, 1, NLy, radices_of(p->ax[1]), twy, MODE_PLAIN, s, gsz);
+  vie_status st = launch_x<V>(true, 0, p->ax[1], p1, count, g.ny, 1, NLy, twy, MODE_PLAIN, s, gsz);
   if (st == VIE_OK) st = dispatch_pass_bz<V>(pp, count, g, twz, s);
-  done = false;
-  if (st == VIE_OK && l1)
-    st = dispatch_x4<V>(false, l1, l2, p3, count, g.ny, 1, NLy, twy, MODE_PLAIN, s, &done, 0, gsz);
-  if (st == VIE_OK && !done)
-    st = launch_x_generic<V>(false, p3, count, g.ny, 1, NLy, radices_of(p->ax[1]), twy, MODE_PLAIN, s, gsz);
+  if (st == VIE_OK) st = launch_x<V>(false, 0, p->ax[1], p3, count, g.ny, 1, NLy, twy, MODE_PLAIN, s, gsz);
   return st;
 }
 
@@ -1384,44 +1241,17 @@ static vie_status run_passes(const vie_plan* p, const PassPtrs<V>& pp, int count
   const int Mx = p->m[0], My = p->m[1], Mz = p->m[2];
   const int NL = 3 * ny * nz;
   const int threads = 256;
-  // generic x passes: lines per block from the shared-memory budget
-  const size_t line_bytes = (size_t)2 * (Mx + 1) * sizeof(V);
-  const size_t tw_bytes = (size_t)Mx * sizeof(V);
-  int lpb = 4;
-  while (lpb > 1 && tw_bytes + lpb * line_bytes > 200 * 1024) lpb >>= 1;
-  const size_t smem_ac = tw_bytes + lpb * line_bytes;
-  if (smem_ac > 220 * 1024) {
-    set_error("Mx = %d too large for the x-pass shared memory", Mx);
-    return VIE_ERR_INVALID;
-  }
   const size_t smem_b = (size_t)(My + Mz + 2 * 3 * Mz * (My + 1)) * sizeof(V);
-  const dim3 blocks_ac((unsigned)((NL + lpb - 1) / lpb), (unsigned)count);
-  int l1 = 0, l2 = 0, a1 = 0, a2 = 0, a3 = 0;
-  x4_factors(Mx, &l1, &l2);
-  x3_factors(Mx, &a1, &a2, &a3);
   bool done = false;
-  vie_status st = VIE_OK;
-  // x passes: three-factor kernels (x_lpb < 0: -x_lpb lines per block; 0:
-  // the default for the forward pass where they exist), else four-step
-  // (x_lpb > 0), else generic
-  if (a1 && p->x_lpb <= 0) {
-    st = dispatch_x3<V>(true, a1, a2, a3, pp, count, nx, ny * nz, NL, twx, mode, s, &done,
-                        p->x_lpb < 0 ? -p->x_lpb : 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done && l1) {
-    st = dispatch_x4<V>(true, l1, l2, pp, count, nx, ny * nz, NL, twx, mode, s, &done, p->x_lpb > 0 ? p->x_lpb : 0,
-                        NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ac));
-    pass_a_kernel<V><<<blocks_ac, threads, smem_ac, s>>>(pp, nx, NL, radices_of(p->ax[0]), twx, lpb, NL);
-    VIE_LAUNCH_CHECK();
-  }
+  vie_status st = launch_x<V>(true, p->x_lpb, p->ax[0], pp, count, nx, ny * nz, NL, twx, mode, s, NL);
+  if (st != VIE_OK) return st;
   PassBGeom g{ny, nz, NL, Mx, My, Mz, p->kf[1], p->kf[2]};
   st = dispatch_pass_b_reg<V>(pp, count, g, twy, twz, s, &done);
   if (st != VIE_OK) return st;
+  if (!done) {
+    st = launch_b_any<V>(pp, count, g, 3, nullptr, 0.0, twy, s, &done);
+    if (st != VIE_OK) return st;
+  }
   if (!done && smem_b > 220 * 1024 && pp.work2[0] && pass_bz_available(Mz)) {
     st = run_split_b<V>(p, pp, count, g, twy, twz, s);
     if (st != VIE_OK) return st;
@@ -1438,27 +1268,7 @@ static vie_status run_passes(const vie_plan* p, const PassPtrs<V>& pp, int count
                                                                                 radices_of(p->ax[2]), twy, twz);
     VIE_LAUNCH_CHECK();
   }
-  done = false;
-  // inverse: three-factor only when chosen (x_lpb_inv < 0) or when no
-  // four-step kernel exists for Mx; the four-step inverse, whose blocks read
-  // 32-byte rows of the transposed workspace, measured faster on the guide
-  if (a1 && (p->x_lpb_inv < 0 || (p->x_lpb_inv == 0 && !l1))) {
-    st = dispatch_x3<V>(false, a1, a2, a3, pp, count, nx, ny * nz, NL, twx, mode, s, &done,
-                        p->x_lpb_inv < 0 ? -p->x_lpb_inv : 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done && l1) {
-    st = dispatch_x4<V>(false, l1, l2, pp, count, nx, ny * nz, NL, twx, mode, s, &done,
-                        p->x_lpb_inv > 0 ? p->x_lpb_inv : 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ac));
-    pass_c_kernel<V><<<blocks_ac, threads, smem_ac, s>>>(pp, nx, ny * nz, NL, radices_of(p->ax[0]), twx, lpb, mode,
-                                                        NL);
-    VIE_LAUNCH_CHECK();
-  }
-  return VIE_OK;
+  return launch_x<V>(false, p->x_lpb_inv, p->ax[0], pp, count, nx, ny * nz, NL, twx, mode, s, NL);
 }
 
 // ---------------------------------------------------------------------------
@@ -1888,37 +1698,16 @@ static vie_status run_jm(vie_plan* p, const V* x, V* y, const V* ghat, const V* 
   pp.work[0] = (V*)p->jm_work;
   pp.ghat[0] = ghat;
   pp.M[0] = Mc;
-  const size_t line_bytes = (size_t)2 * (Mx + 1) * sizeof(V);
-  const size_t tw_bytes = (size_t)Mx * sizeof(V);
-  int lpb = 4;
-  while (lpb > 1 && tw_bytes + lpb * line_bytes > 200 * 1024) lpb >>= 1;
-  const size_t smem_ac = tw_bytes + lpb * line_bytes;
-  if (smem_ac > 220 * 1024) {
-    set_error("Mx = %d too large for the x-pass shared memory", Mx);
-    return VIE_ERR_INVALID;
-  }
-  const dim3 blocks_ac((unsigned)((NL + lpb - 1) / lpb), 1);
-  int l1 = 0, l2 = 0, a1 = 0, a2 = 0, a3 = 0;
-  x4_factors(Mx, &l1, &l2);
-  x3_factors(Mx, &a1, &a2, &a3);
   bool done = false;
-  vie_status st = VIE_OK;
-  if (a1) {
-    st = dispatch_x3<V>(true, a1, a2, a3, pp, 1, nx, NL, NL, twx, mode, s, &done, 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done && l1) {
-    st = dispatch_x4<V>(true, l1, l2, pp, 1, nx, NL, NL, twx, mode, s, &done, 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ac));
-    pass_a_kernel<V><<<blocks_ac, 256, smem_ac, s>>>(pp, nx, NL, radices_of(p->ax[0]), twx, lpb, NL);
-    VIE_LAUNCH_CHECK();
-  }
+  vie_status st = launch_x<V>(true, 0, p->ax[0], pp, 1, nx, NL, NL, twx, mode, s, NL);
+  if (st != VIE_OK) return st;
   PassBGeom g{ny, nz, NL, Mx, My, Mz, p->kf[1], p->kf[2]};
   st = dispatch_pass_b_reg_jm<V>((V*)p->jm_work, ghat, chat, g, twy, twz, p->kappa, s, &done);
   if (st != VIE_OK) return st;
+  if (!done) {
+    st = launch_b_any<V>(pp, 1, g, 6, chat, p->kappa, twy, s, &done);
+    if (st != VIE_OK) return st;
+  }
   if (!done && smem_b <= 220 * 1024) {
     VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_jm_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
     pass_b_jm_kernel<V><<<(unsigned)Mx, 256, smem_b, s>>>((V*)p->jm_work, ghat, chat, g, radices_of(p->ax[1]),
@@ -1934,21 +1723,7 @@ static vie_status run_jm(vie_plan* p, const V* x, V* y, const V* ghat, const V* 
                                                                  twz, p->kappa);
     VIE_LAUNCH_CHECK();
   }
-  done = false;
-  if (a1) {
-    st = dispatch_x3<V>(false, a1, a2, a3, pp, 1, nx, NL, NL, twx, mode, s, &done, 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done && l1) {
-    st = dispatch_x4<V>(false, l1, l2, pp, 1, nx, NL, NL, twx, mode, s, &done, 0, NL);
-    if (st != VIE_OK) return st;
-  }
-  if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ac));
-    pass_c_kernel<V><<<blocks_ac, 256, smem_ac, s>>>(pp, nx, NL, NL, radices_of(p->ax[0]), twx, lpb, mode, NL);
-    VIE_LAUNCH_CHECK();
-  }
-  return VIE_OK;
+  return launch_x<V>(false, 0, p->ax[0], pp, 1, nx, NL, NL, twx, mode, s, NL);
 }
 
 vie_status jm_matvec_impl(vie_plan* p, const void* x, void* y, int dtype, int mode, cudaStream_t s) {

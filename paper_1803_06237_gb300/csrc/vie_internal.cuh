@@ -55,6 +55,21 @@ template <typename V> __host__ __device__ __forceinline__ V mulc(V a, V b) {
   V r; r.x = a.x * b.x + a.y * b.y; r.y = a.y * b.x - a.x * b.y; return r;
 }
 template <typename V, typename R> __host__ __device__ __forceinline__ V scale(V a, R s) { V r; r.x = a.x * s; r.y = a.y * s; return r; }
+// complex64 sums as one packed instruction: the FP32 rate is that of the
+// scalar forms, but half as many instructions issue (the FFT passes are bound
+// by issue slots).
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+// a * s + c for a real s; (sx, sy) scale the two parts
+__device__ __forceinline__ float2 fma2(float2 a, float s, float2 c) { return __ffma2_rn(a, make_float2(s, s), c); }
+__device__ __forceinline__ float2 fma2(float2 a, float sx, float sy, float2 c) { return __ffma2_rn(a, make_float2(sx, sy), c); }
+// a (c + i s): two products and one packed multiply-add
+__device__ __forceinline__ float2 mul_cs(float2 a, float c, float s) { return fma2(a, c, make_float2(-a.y * s, a.x * s)); }
+__device__ __forceinline__ double2 mul_cs(double2 a, double c, double s) {
+  return make_double2(a.x * c - a.y * s, a.x * s + a.y * c);
+}
+// the difference with its parts exchanged: -i d = swapped * (1, -1), +i d = swapped * (-1, 1)
+__device__ __forceinline__ float2 sub_swapped(float2 a, float2 b) { return make_float2(a.y - b.y, a.x - b.x); }
 // -i * a  and  +i * a
 template <typename V> __host__ __device__ __forceinline__ V mul_mi(V a) { V r; r.x = a.y; r.y = -a.x; return r; }
 template <typename V> __host__ __device__ __forceinline__ V mul_pi(V a) { V r; r.x = -a.y; r.y = a.x; return r; }
@@ -117,8 +132,7 @@ inline Radices radices_of(const AxisPlan& a) {
 
 bool factor_length(int len, AxisPlan* out);   // radices from {4, 2, 3, 5}
 bool factor_length_any(int len, AxisPlan* out);   // 4, 2, 3, 5, then larger primes (generic stages)
-void x4_factors(int mx, int* l1, int* l2);    // compiled four-step split of Mx, or (0, 0)
-void x3_factors(int mx, int* l1, int* l2, int* l3);   // compiled three-factor split of Mx, or zeros
+bool x_lines_compiled(int nx, int mx);        // x-pass kernels compiled for lines of nx values into mx
 int smooth_size_at_least(int n);               // smallest 5-smooth >= n
 
 // ---------------------------------------------------------------------------
