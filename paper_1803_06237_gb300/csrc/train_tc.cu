@@ -25,7 +25,12 @@
 // (z + dz - 1, y + dy - 1), planar, the TMA zero-filling rows outside the
 // grid).  Nine accumulators of 128 x C in tensor memory collect a CTA's
 // chunks; the epilogue writes them as per-CTA partial sums, reduced by
-// dw_reduce_kernel into the FP32 gradient.
+// dw_reduce_kernel into the FP32 gradient.  Nothing in the chain of input
+// gradients needs a weight gradient, so the eight layers' operands, GEMMs and
+// reductions run as three launches after it, each layer with its share of one
+// CTA per SM: as three launches per layer they took 303 of 520 us a sample
+// (160 x 40 x 11), most of it the ends of short kernels (a GEMM of 14 CTAs
+// with four chunks each takes 14 us, one of 152 with nine takes 22).
 #include <cuda_bf16.h>
 #include <stdio.h>
 
@@ -42,32 +47,57 @@ constexpr int kDwMinChunks = 4;    // chunks per CTA at least, where the level a
 // ---------------------------------------------------------------------------
 // planar operands of the weight-gradient GEMM
 // ---------------------------------------------------------------------------
-// The two operands in one launch (grid.x = 2 x the chunks per row; blocks
-// below nxc write A, the others B), one block per (64-position chunk, y, z);
-// rows are `plane` elements apart (the level-0 plane at every level):
+// One layer of the weight-gradient launches.
+struct DwLayer {
+  const __nv_bfloat16* g;    // gradient of the pre-activation, NPo channels
+  const __nv_bfloat16* in;   // layer input, C channels
+  __nv_bfloat16* A;          // planar operands, rows `plane` elements apart
+  __nv_bfloat16* B;
+  float* gb;                 // bias gradient
+  float* gw;                 // weight gradient
+  size_t plane;
+  Dims d;
+  int NPo, co, ci, C;
+  int nxp, nxc;              // padded row, chunks per row
+  int block0;                // first block of the operand launch
+  int cta0, ctas;            // CTAs of the GEMM
+};
+struct DwArgs {
+  DwLayer l[kNumLayers];
+  int stages;
+  float* partial;            // [CTA][27][32][C], CTAs 27 x 32 x 32 apart
+  int* bad;
+};
+
+// Operand blocks: per layer and (z, y) row 2 nxc blocks, the first nxc write
+// A, the others B, each for 64 positions:
 //   A[dx * 32 + o][z][y][x] = g[z][y][x - dx + 1][o] for dx < 3, o < NPo and
 //     0 <= x - dx + 1 < nx, x < nx; 0 elsewhere (rows 96..127 are zeroed
 //     once when the buffer is laid out and never written);
 //   B[c][z][y][x] = in[z][y][x][c] for x < nx, 0 for nx <= x < nxp;
 // and the A blocks add their chunk's sum of g over positions to the bias
-// gradient gb[o] (o < co).
-__global__ void __launch_bounds__(256) dw_operands_kernel(const __nv_bfloat16* __restrict__ g, int NPo, int co,
-                                                          const __nv_bfloat16* __restrict__ in, int C, Dims d,
-                                                          int nxp, int nxc, size_t plane, __nv_bfloat16* __restrict__ A,
-                                                          __nv_bfloat16* __restrict__ B, float* __restrict__ gb) {
+// gradient gb[o] (o < co).  Rows are written 16 bytes a thread.
+__global__ void __launch_bounds__(256) dw_operands_kernel(const __grid_constant__ DwArgs args) {
   __shared__ __nv_bfloat16 t[kDwChunk + 2][33];
   __shared__ float bsum[8][33];
-  const bool isA = (int)blockIdx.x < nxc;
-  const int x0 = (isA ? blockIdx.x : blockIdx.x - nxc) * kDwChunk, y = blockIdx.y, z = blockIdx.z;
-  const size_t row = (size_t)z * d.ny + y;
-  const size_t base = row * nxp + x0;
+  int li = kNumLayers - 1;
+  while (li > 0 && (int)blockIdx.x < args.l[li].block0) --li;
+  const DwLayer& L = args.l[li];
+  const Dims d = L.d;
+  const int id = blockIdx.x - L.block0, per = 2 * L.nxc;
+  const size_t row = id / per;                        // z ny + y
+  const int xb = id - (int)row * per;
+  const bool isA = xb < L.nxc;
+  const int x0 = (isA ? xb : xb - L.nxc) * kDwChunk;
+  const size_t base = row * L.nxp + x0;
+  const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
   if (isA) {
     float acc = 0.f;   // thread (j, o) sums g over its positions j = tid >> 5, + 8, ...
     for (int i = threadIdx.x; i < (kDwChunk + 2) * 32; i += blockDim.x) {
       const int j = i >> 5, o = i & 31;
       const int x = x0 - 1 + j;
-      __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-      if (o < NPo && x >= 0 && x < d.nx) v = g[(row * d.nx + x) * NPo + o];
+      __nv_bfloat16 v = zero;
+      if (o < L.NPo && x >= 0 && x < d.nx) v = L.g[(row * d.nx + x) * L.NPo + o];
       t[j][o] = v;
       if (j >= 1 && j <= kDwChunk) acc += __bfloat162float(v);   // positions x0 .. x0 + 63 of this chunk
     }
@@ -76,44 +106,40 @@ __global__ void __launch_bounds__(256) dw_operands_kernel(const __nv_bfloat16* _
     if (threadIdx.x < 32) {
       float sum = 0.f;
       for (int k = 0; k < 8; ++k) sum += bsum[k][threadIdx.x];
-      if (threadIdx.x < co) atomicAdd(gb + threadIdx.x, sum);
-    }
-    for (int i = threadIdx.x; i < 96 * kDwChunk; i += blockDim.x) {
-      const int r = i / kDwChunk, xl = i - r * kDwChunk;
-      const int dx = r >> 5, o = r & 31;
-      __nv_bfloat16 v = __float2bfloat16_rn(0.f);
-      if (x0 + xl < d.nx) v = t[xl - dx + 2][o];
-      A[r * plane + base + xl] = v;
+      if (threadIdx.x < L.co) atomicAdd(L.gb + threadIdx.x, sum);
     }
   } else {
-    for (int i = threadIdx.x; i < kDwChunk * C; i += blockDim.x) {
-      const int j = i / C, c = i - j * C;
+    for (int i = threadIdx.x; i < kDwChunk * L.C; i += blockDim.x) {
+      const int j = i / L.C, c = i - j * L.C;
       const int x = x0 + j;
-      t[j][c] = x < d.nx ? in[(row * d.nx + x) * C + c] : __float2bfloat16_rn(0.f);
+      t[j][c] = x < d.nx ? L.in[(row * d.nx + x) * L.C + c] : zero;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < C * kDwChunk; i += blockDim.x) {
-      const int c = i / kDwChunk, xl = i - c * kDwChunk;
-      B[c * plane + base + xl] = t[xl][c];
-    }
+  }
+  // 8 positions a thread of row r: t[x - dx + 2][o] (A), t[x][c] (B)
+  const int rows = isA ? 96 : L.C;
+  __nv_bfloat16* out = isA ? L.A : L.B;
+  for (int i = threadIdx.x; i < rows * (kDwChunk / 8); i += blockDim.x) {
+    const int r = i >> 3, xl = (i & 7) * 8;
+    const int c = r & 31, shift = isA ? 2 - (r >> 5) : 0;
+    __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = x0 + xl + k < d.nx ? t[xl + k + shift][c] : zero;
+    *reinterpret_cast<uint4*>(out + r * L.plane + base + xl) = *reinterpret_cast<const uint4*>(v);
   }
 }
 
 // ---------------------------------------------------------------------------
 // weight-gradient GEMM on the tensor cores
 // ---------------------------------------------------------------------------
-struct DwArgs {
-  Dims d;
-  int nxc;            // chunks per (z, y) row
-  int stages;
-  float* partial;     // [gridDim.x][27][32][C]
-  int* bad;
+struct DwMaps {
+  CUtensorMap a[kNumLayers], b[kNumLayers];
 };
 
+// One CTA's share of a layer: its chunks into the CTA's partial sums.
 template <int C>
-__global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_constant__ CUtensorMap tmA,
-                                                              const __grid_constant__ CUtensorMap tmB,
-                                                              const DwArgs a) {
+__device__ __forceinline__ void dw_gemm(const CUtensorMap& tmA, const CUtensorMap& tmB, const DwLayer& L, int cta,
+                                        int stages, float* partial, int* bad) {
   constexpr uint32_t ABYTES = 128 * 128;          // 128 rows x 64 positions (BF16)
   constexpr uint32_t BBYTES = C * 128;            // C rows x 64 positions
   constexpr uint32_t SBYTES = ABYTES + 9 * BBYTES;
@@ -121,17 +147,17 @@ __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_const
   constexpr uint32_t IDESC = tc::idesc_bf16_f32(128, C);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  const uint32_t S = (uint32_t)a.stages;
+  const uint32_t S = (uint32_t)stages;
   uint64_t* full = (uint64_t*)(base + S * SBYTES);
   uint64_t* empty = full + kDwMaxStages;
   uint64_t* done = empty + kDwMaxStages;
   uint32_t* tslot = (uint32_t*)(done + 1);
   volatile int* abort = (volatile int*)(tslot + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long nchunks = (long)a.d.nz * a.d.ny * a.nxc;
-  // balanced contiguous ranges: every CTA has at least one chunk (grid <= nchunks)
-  const long k0 = (long)blockIdx.x * nchunks / gridDim.x;
-  const long k1 = (long)(blockIdx.x + 1) * nchunks / gridDim.x;
+  const long nchunks = (long)L.d.nz * L.d.ny * L.nxc;
+  // balanced contiguous ranges: every CTA has at least one chunk (ctas <= nchunks)
+  const long k0 = (long)cta * nchunks / L.ctas;
+  const long k1 = (long)(cta + 1) * nchunks / L.ctas;
 
   if (threadIdx.x == 0) {
     for (uint32_t i = 0; i < S; ++i) {
@@ -156,9 +182,9 @@ __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_const
     tc::prefetch_tensormap(&tmB);
     uint32_t it = 0;
     for (long k = k0; k < k1 && !*abort; ++k, ++it) {
-      const int xc = (int)(k % a.nxc);
-      const long row = k / a.nxc;
-      const int y = (int)(row % a.d.ny), z = (int)(row / a.d.ny);
+      const int xc = (int)(k % L.nxc);
+      const long row = k / L.nxc;
+      const int y = (int)(row % L.d.ny), z = (int)(row / L.d.ny);
       const uint32_t stage = it % S, round = it / S;
       if (!tc::mbar_wait(&empty[stage], (round & 1) ^ 1, abort)) break;
       tc::mbar_arrive_expect_tx(&full[stage], SBYTES);
@@ -213,14 +239,14 @@ __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_const
         float v[C];
         if constexpr (C == 32) tc::tmem_ld32(tmem + lane_base + (uint32_t)(t * C), v);
         else tc::tmem_ld16(tmem + lane_base + (uint32_t)(t * C), v);
-        float4* dst = reinterpret_cast<float4*>(a.partial + (((size_t)blockIdx.x * 27 + 3 * t + q) * 32 + lane) * C);
+        float4* dst = reinterpret_cast<float4*>(partial + ((size_t)(3 * t + q) * 32 + lane) * C);
 #pragma unroll
         for (int i = 0; i < C / 4; ++i) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
       }
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && *abort) atomicExch(a.bad, 2);
+  if (threadIdx.x == 0 && *abort) atomicExch(bad, 2);
   if (warp == 1) {
     __syncwarp();
     tc::fence_after_sync();
@@ -228,20 +254,35 @@ __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_const
   }
 }
 
-// grad[(o ci + c) 27 + t] += sum_b partial[b][t][o][c]: thread i runs over
-// the partial layout (t, o, c) so that the reads of every b are coalesced,
-// blockIdx.y takes every gridDim.y-th b and adds its share atomically
-__global__ void dw_reduce_kernel(const float* __restrict__ partial, int nb, int C, int ci, int co,
-                                 float* __restrict__ grad) {
-  const int n = 27 * 32 * C;
+constexpr size_t kDwPartial = (size_t)27 * 32 * 32;   // floats of a CTA's partial sums
+
+__global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_constant__ DwMaps maps,
+                                                              const __grid_constant__ DwArgs args) {
+  int li = kNumLayers - 1;
+  while (li > 0 && (int)blockIdx.x < args.l[li].cta0) --li;
+  const DwLayer& L = args.l[li];
+  const int cta = blockIdx.x - L.cta0;
+  float* partial = args.partial + blockIdx.x * kDwPartial;
+  if (L.C == 32) dw_gemm<32>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
+  else dw_gemm<16>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
+}
+
+// gw[(o ci + c) 27 + t] += sum_b partial[b][t][o][c] over the layer's CTAs
+// (blockIdx.y): thread i runs over the partial layout (t, o, c) so that the
+// reads of every b are coalesced, blockIdx.z takes every gridDim.z-th b and
+// adds its share atomically
+__global__ void dw_reduce_kernel(const __grid_constant__ DwArgs args) {
+  const DwLayer& L = args.l[blockIdx.y];
+  const int n = 27 * 32 * L.C;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int c = i % C, o = (i / C) % 32, t = i / (32 * C);
-  if (o >= co || c >= ci) return;
+  if (i >= n || (int)blockIdx.z >= L.ctas) return;
+  const int c = i % L.C, o = (i / L.C) % 32, t = i / (32 * L.C);
+  if (o >= L.co || c >= L.ci) return;
+  const float* partial = args.partial + (size_t)L.cta0 * kDwPartial;
   float acc = 0.f;
 #pragma unroll 4
-  for (int b = blockIdx.y; b < nb; b += gridDim.y) acc += partial[(size_t)b * n + i];
-  atomicAdd(grad + (o * ci + c) * 27 + t, acc);
+  for (int b = blockIdx.z; b < L.ctas; b += gridDim.z) acc += partial[(size_t)b * kDwPartial + i];
+  atomicAdd(L.gw + (o * L.ci + c) * 27 + t, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -399,21 +440,23 @@ struct TcTrain {
   // backward: dY (16 channels), per layer the gradient of its pre-activation
   // dpre[l], the input gradients of the decoders (ddecin_l) and encoders (da_l)
   __nv_bfloat16 *dY = nullptr, *dpre[kNumLayers] = {}, *ddecin[3] = {}, *da[4] = {};
-  __nv_bfloat16 *Apl = nullptr, *Bpl = nullptr;   // planar GEMM operands (level 0 size)
-  size_t plane0 = 0;                               // their row stride (elements)
+  __nv_bfloat16 *Apl[kNumLayers] = {}, *Bpl[kNumLayers] = {};   // planar GEMM operands of each layer
+  size_t plane[kNumLayers] = {};                                // their row strides (elements)
   float* Yf = nullptr;                             // network output [V0][16]
   size_t yf_cap = 0;
-  float* partial = nullptr;                        // [sms][27][32][32]
+  float* partial = nullptr;                        // [sms] partial sums of kDwPartial
   double* norm = nullptr;                          // kTcNormBlocks + 1 partial sums of |r|^2, then loss sums
   int bxf[kNumLayers], byf[kNumLayers];            // forward tiles
   int bxb[kNumLayers], byb[kNumLayers];            // backward-data tiles
   CUtensorMap mA[kNumLayers], mW[kNumLayers];      // forward input / weights
   CUtensorMap mG[kNumLayers], mWf[kNumLayers];     // backward-data input (the layer's output gradient) / weights
-  CUtensorMap mPa[kNumLayers], mPb[kNumLayers];    // weight-gradient operands
+  DwMaps mP;                                       // weight-gradient operands
   int sms = 0, smem_optin = 0;
   const void* wpack_enc = nullptr;                 // weights the maps mW / mWf point at
   const void* wpackf_enc = nullptr;
 };
+
+constexpr size_t kMapAlign = 128;   // elements: operand buffers start on 256 bytes
 
 static int nxp_of(int nx) { return (nx + kDwChunk - 1) / kDwChunk * kDwChunk; }
 
@@ -437,7 +480,7 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
     VIE_CUDA_TRY(cudaDeviceGetAttribute(&T->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     if (!T->partial) {
       float* buf = nullptr;
-      VIE_CUDA_TRY(cudaMalloc((void**)&buf, (size_t)T->sms * 27 * 32 * 32 * sizeof(float)));
+      VIE_CUDA_TRY(cudaMalloc((void**)&buf, (size_t)T->sms * kDwPartial * sizeof(float)));
       T->partial = buf;
     }
     if (!T->norm) {
@@ -456,8 +499,11 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
     for (int l = 1; l < 4; ++l) need += 32 * T->L[l].vox();       // a_l
     for (int l = 0; l < 3; ++l) need += 32 * T->L[l].vox() * 3;   // decin_l, u_l, ddecin_l
     for (int l = 0; l < kNumLayers; ++l) need += 32 * T->L[kLayerLevel[l]].vox();   // dpre
-    const size_t plane0 = (size_t)T->L[0].nz * T->L[0].ny * nxp_of(T->L[0].nx);
-    need += 128 * plane0 + 32 * plane0;                           // Apl, Bpl
+    for (int l = 0; l < kNumLayers; ++l) {                        // Apl, Bpl
+      const Dims d = T->L[kLayerLevel[l]];
+      T->plane[l] = (size_t)d.nz * d.ny * nxp_of(d.nx);
+      need += (128 + tc_cpad(kLayerDefs[l].ci)) * T->plane[l] + 2 * kMapAlign;
+    }
     if (need > T->cap) {
       cudaFree(T->ws);
       T->ws = nullptr;
@@ -491,11 +537,13 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
       T->ddecin[l] = take(32 * T->L[l].vox());
     }
     for (int l = 0; l < kNumLayers; ++l) T->dpre[l] = take(32 * T->L[kLayerLevel[l]].vox());
-    T->Apl = take(128 * plane0);
-    T->Bpl = take(32 * plane0);
-    T->plane0 = plane0;
-    // rows 96..127 of A (no dx block) stay zero
-    VIE_CUDA_TRY(cudaMemset(T->Apl + 96 * plane0, 0, 32 * plane0 * sizeof(__nv_bfloat16)));
+    for (int l = 0; l < kNumLayers; ++l) {
+      p = T->ws + ((p - T->ws) + kMapAlign - 1) / kMapAlign * kMapAlign;
+      T->Apl[l] = take(128 * T->plane[l]);
+      T->Bpl[l] = take(tc_cpad(kLayerDefs[l].ci) * T->plane[l]);
+      // rows 96..127 of A (no dx block) stay zero
+      VIE_CUDA_TRY(cudaMemset(T->Apl[l] + 96 * T->plane[l], 0, 32 * T->plane[l] * sizeof(__nv_bfloat16)));
+    }
     // forward maps: the inputs of enc0..enc3, dec2, dec1, dec0, out
     const __nv_bfloat16* in[kNumLayers] = {T->X, T->a[1], T->a[2], T->a[3], T->decin[2], T->decin[1], T->decin[0],
                                            T->u[0]};
@@ -511,8 +559,8 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
                          T->byb[l]);
       if (st != VIE_OK) return st;
       const int nxp = nxp_of(d.nx);
-      if ((st = tc_encode_planar(&T->mPa[l], T->Apl, 128, d, nxp, plane0)) != VIE_OK) return st;
-      if ((st = tc_encode_planar(&T->mPb[l], T->Bpl, tc_cpad(kLayerDefs[l].ci), d, nxp, plane0)) != VIE_OK)
+      if ((st = tc_encode_planar(&T->mP.a[l], T->Apl[l], 128, d, nxp, T->plane[l])) != VIE_OK) return st;
+      if ((st = tc_encode_planar(&T->mP.b[l], T->Bpl[l], tc_cpad(kLayerDefs[l].ci), d, nxp, T->plane[l])) != VIE_OK)
         return st;
     }
     T->n[0] = n[0];
@@ -539,51 +587,70 @@ static unsigned ew_grid(size_t n) {
   return (unsigned)(b < 152 * 16 ? (b ? b : 1) : 152 * 16);
 }
 
-// weight and bias gradients of `layer` from its pre-activation gradient g
-// (NPo channels) and its input `in` (tc_cpad(ci) channels), added to grad
-static vie_status weight_grad_tc(const TcTrain* T, const TcTrainParams& P, int layer, const __nv_bfloat16* g,
-                                 const __nv_bfloat16* in, cudaStream_t s) {
-  const Dims d = T->L[kLayerLevel[layer]];
-  const int ci = kLayerDefs[layer].ci, co = kLayerDefs[layer].co;
-  const int C = tc_cpad(ci), NPo = tc_npad(co);
-  const int nxp = nxp_of(d.nx);
-  const int nxc = nxp / kDwChunk;
-  dw_operands_kernel<<<dim3((unsigned)(2 * nxc), (unsigned)d.ny, (unsigned)d.nz), 256, 0, s>>>(
-      g, NPo, co, in, C, d, nxp, nxc, T->plane0, T->Apl, T->Bpl, P.grad + layer_b_off(layer));
-  VIE_LAUNCH_CHECK();
-  constexpr size_t kSB32 = 128 * 128 + 9 * 32 * 128, kSB16 = 128 * 128 + 9 * 16 * 128;
+// Weight and bias gradients of every layer from its pre-activation gradient
+// (NPo channels) and its input (tc_cpad(ci) channels), added to grad.
+static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, cudaStream_t s) {
+  const __nv_bfloat16* in[kNumLayers] = {T->X, T->a[1], T->a[2], T->a[3], T->decin[2], T->decin[1], T->decin[0],
+                                         T->u[0]};
+  DwArgs a{};
+  long chunks[kNumLayers], total = 0, want = 0;
+  unsigned blocks = 0;
+  for (int l = 0; l < kNumLayers; ++l) {
+    DwLayer& L = a.l[l];
+    L.d = T->L[kLayerLevel[l]];
+    L.g = l == OUTL ? T->dY : T->dpre[l];
+    L.in = in[l];
+    L.A = T->Apl[l];
+    L.B = T->Bpl[l];
+    L.gb = P.grad + layer_b_off(l);
+    L.gw = P.grad + layer_w_off(l);
+    L.plane = T->plane[l];
+    L.ci = kLayerDefs[l].ci;
+    L.co = kLayerDefs[l].co;
+    L.C = tc_cpad(L.ci);
+    L.NPo = tc_npad(L.co);
+    L.nxp = nxp_of(L.d.nx);
+    L.nxc = L.nxp / kDwChunk;
+    L.block0 = (int)blocks;
+    blocks += (unsigned)(2 * L.nxc * L.d.ny * L.d.nz);
+    chunks[l] = (long)L.d.nz * L.d.ny * L.nxc;
+    total += chunks[l];
+    want += (chunks[l] + kDwMinChunks - 1) / kDwMinChunks;
+  }
+  // one CTA per SM at most, each layer's share by its chunks: one each, then
+  // to the layer with the most chunks a CTA
+  const int ctas = (int)(want < T->sms ? want : T->sms);
+  for (int l = 0; l < kNumLayers; ++l) a.l[l].ctas = 1;
+  for (int k = kNumLayers; k < ctas; ++k) {
+    int most = 0;
+    for (int l = 1; l < kNumLayers; ++l)
+      if (chunks[l] * a.l[most].ctas > chunks[most] * a.l[l].ctas) most = l;
+    if (a.l[most].ctas >= chunks[most]) break;
+    ++a.l[most].ctas;
+  }
+  int used = 0;
+  for (int l = 0; l < kNumLayers; ++l) {
+    a.l[l].cta0 = used;
+    used += a.l[l].ctas;
+  }
+  constexpr size_t SB = 128 * 128 + 9 * 32 * 128;
   const size_t fixed = 1024 + 2 * kDwMaxStages * 8 + 64;
-  const size_t SB = C == 32 ? kSB32 : kSB16;
   int stages = (int)(((size_t)T->smem_optin - fixed) / SB);
   if (stages > kDwMaxStages) stages = kDwMaxStages;
-  if (stages < 2) {
-    set_error("weight-gradient GEMM: %zu B per stage does not fit", SB);
+  if (stages < 2 || used > T->sms) {
+    set_error("weight-gradient GEMM: %zu B per stage do not fit, or %d CTAs on %d SMs", SB, used, T->sms);
     return VIE_ERR_INVALID;
   }
-  const size_t smem = fixed + (size_t)stages * SB;
-  DwArgs a{};
-  a.d = d;
-  a.nxc = nxp / kDwChunk;
   a.stages = stages;
   a.partial = T->partial;
   a.bad = P.bad;
-  // at least kDwMinChunks chunks per CTA where the level is small: fewer
-  // partial sums to write and reduce
-  const long nchunks = (long)d.nz * d.ny * a.nxc;
-  long want = (nchunks + kDwMinChunks - 1) / kDwMinChunks;
-  if (want < 1) want = 1;
-  const int nb = (int)(want < T->sms ? want : T->sms);
-  if (C == 32) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(dw_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dw_tc_kernel<32><<<nb, kDwThreads, smem, s>>>(T->mPa[layer], T->mPb[layer], a);
-  } else {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(dw_tc_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dw_tc_kernel<16><<<nb, kDwThreads, smem, s>>>(T->mPa[layer], T->mPb[layer], a);
-  }
+  const size_t smem = fixed + (size_t)stages * SB;
+  dw_operands_kernel<<<blocks, 256, 0, s>>>(a);
   VIE_LAUNCH_CHECK();
-  const int nred = 27 * 32 * C, slices = nb < 16 ? nb : 16;
-  dw_reduce_kernel<<<dim3((unsigned)((nred + 255) / 256), (unsigned)slices), 256, 0, s>>>(
-      T->partial, nb, C, ci, co, P.grad + layer_w_off(layer));
+  VIE_CUDA_TRY(cudaFuncSetAttribute(dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  dw_tc_kernel<<<used, kDwThreads, smem, s>>>(T->mP, a);
+  VIE_LAUNCH_CHECK();
+  dw_reduce_kernel<<<dim3((unsigned)(kDwPartial / 256), kNumLayers, 8), 256, 0, s>>>(a);
   VIE_LAUNCH_CHECK();
   return VIE_OK;
 }
@@ -643,12 +710,10 @@ vie_status tc_train_accumulate(TcTrain** pt, const TcTrainParams& P, const int n
   };
   const Dims* L = T->L;
   // output layer: input u_0 = relu(dec0)
-  if ((st = weight_grad_tc(T, P, OUTL, T->dY, T->u[0], s)) != VIE_OK) return st;
   if ((st = bwd(OUTL, T->dpre[DEC0], T->u[0])) != VIE_OK) return st;
   // decoders: input decin_l = up(u_{l+1}) + h_l (u_3 = h_3)
   for (int l = 0; l <= 2; ++l) {
     const int layer = DEC0 - l;   // dec0, dec1, dec2
-    if ((st = weight_grad_tc(T, P, layer, T->dpre[layer], T->decin[l], s)) != VIE_OK) return st;
     if ((st = bwd(layer, T->ddecin[l], nullptr)) != VIE_OK) return st;
     const int coarse_layer = l == 2 ? ENC3 : layer - 1;      // producer of the coarse tensor
     const __nv_bfloat16* coarse = l == 2 ? T->h[3] : T->u[l + 1];
@@ -657,16 +722,14 @@ vie_status tc_train_accumulate(TcTrain** pt, const TcTrainParams& P, const int n
     VIE_LAUNCH_CHECK();
   }
   // encoders: input a_l = pool(h_{l-1}) (X for enc0); h_{l-1} also feeds decin_{l-1}
-  for (int l = 3; l >= 0; --l) {
+  for (int l = 3; l >= 1; --l) {
     const int layer = ENC0 + l;
-    const __nv_bfloat16* in = l == 0 ? T->X : T->a[l];
-    if ((st = weight_grad_tc(T, P, layer, T->dpre[layer], in, s)) != VIE_OK) return st;
-    if (l == 0) break;
     if ((st = bwd(layer, T->da[l], nullptr)) != VIE_OK) return st;
     poolback_mask_kernel<<<ew_grid(L[l - 1].vox() * 4), 256, 0, s>>>(T->ddecin[l - 1], T->da[l], L[l], T->h[l - 1],
                                                                       L[l - 1], T->dpre[ENC0 + l - 1]);
     VIE_LAUNCH_CHECK();
   }
+  if ((st = weight_grads_tc(T, P, s)) != VIE_OK) return st;
   if (loss) {
     double h[3] = {0, 0, 0};
     VIE_CUDA_TRY(cudaMemcpyAsync(h, sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
