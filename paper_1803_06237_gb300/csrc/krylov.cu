@@ -843,56 +843,58 @@ __device__ void coop_reduce(const ProbK* __restrict__ P, int count, const int* s
 }
 
 // The end of the FP64 least-squares step of column j: thread 0 forms the new
-// rotation O_j on (r_j, h_{j+1,j} = hn), updates g and the status, and Q's
+// rotation O_j on (r_j, h_{j+1,j} = sqrt(hn2)), updates g and the status, and Q's
 // rows j and j + 1 are replaced by O_j applied to (row j, e_{j+1}).  r: the
 // column with the earlier rotations applied (shared memory, j + 2 entries).
-__device__ void lsq_column(const ProbK& q, int j, int ldh, double hn, double inv, double2* r) {
+__device__ void lsq_column(const ProbK& q, int j, int ldh, double hn2, double2* r) {
   __shared__ double2 rot[2];   // (c, 0), s
   const int ldq = ldh;
   __syncthreads();
   if (threadIdx.x == 0) {
+    // one thread's FP64 chain ends every step: reciprocal square roots in
+    // place of hypot and divisions, |g_{j+1}| = |g_j| |s| from the last |g_j|
     SolveStatus* st = q.st;
-    const double2 a = r[j], b = make_double2(hn, 0.0);
-    const double aa = hypot(a.x, a.y), ab = hypot(b.x, b.y);
-    const double den = hypot(aa, ab);
-    double c;
+    const double resid = st->resid, beta = st->beta, target = st->target;
+    const double2 gj = q.g[j], a = r[j];
+    const double aa2 = a.x * a.x + a.y * a.y;
+    const double rhn = rsqrt(hn2), hn = hn2 > 0.0 ? hn2 * rhn : hn2;
+    double c, sn;              // |s|
     double2 s;
-    if (den == 0.0) {
-      c = 1.0; s = make_double2(0.0, 0.0);
-    } else if (aa == 0.0) {
-      c = 0.0; s = make_double2(1.0, 0.0);
+    if (aa2 + hn2 == 0.0) {
+      c = 1.0; sn = 0.0; s = make_double2(0.0, 0.0);
+    } else if (aa2 == 0.0) {
+      c = 0.0; sn = 1.0; s = make_double2(1.0, 0.0);
     } else {
-      c = aa / den;
-      const double2 ua = make_double2(a.x / aa, a.y / aa);
-      s = make_double2((ua.x * b.x + ua.y * b.y) / den, (ua.y * b.x - ua.x * b.y) / den);
+      const double ra = rsqrt(aa2), rd = rsqrt(aa2 + hn2);
+      c = aa2 * ra * rd;
+      sn = hn * rd;
+      s = make_double2(a.x * ra * sn, a.y * ra * sn);   // (a / |a|) h_{j+1,j} / den
     }
     q.cs[j] = c;
     q.sn[j] = s;
     rot[0] = make_double2(c, 0.0);
     rot[1] = s;
-    r[j] = make_double2(c * a.x + (s.x * b.x - s.y * b.y), c * a.y + (s.x * b.y + s.y * b.x));
+    r[j] = make_double2(c * a.x + s.x * hn, c * a.y + s.y * hn);
     r[j + 1] = make_double2(0.0, 0.0);
-    const double2 gj = q.g[j];
-    const double2 g1 = make_double2(-(s.x * gj.x + s.y * gj.y), -(s.x * gj.y - s.y * gj.x));
-    q.g[j + 1] = g1;
+    q.g[j + 1] = make_double2(-(s.x * gj.x + s.y * gj.y), -(s.x * gj.y - s.y * gj.x));
     q.g[j] = make_double2(c * gj.x, c * gj.y);
-    const double res = hypot(g1.x, g1.y);
+    const double res = resid * sn;
     st->j = j + 1;
     st->resid = res;
-    if (!(isfinite(hn) && isfinite(res))) {
+    if (!(isfinite(hn) && isfinite(res) && isfinite(c))) {
       st->breakdown = 1;
       st->active = 0;
       st->j = j;
     } else {
-      if (res <= st->target) {
+      if (res <= target) {
         st->converged = 1;
         st->active = 0;
       }
-      if (hn <= 1e-300 || hn <= 1e-14 * st->beta) {
+      if (hn <= 1e-300 || hn <= 1e-14 * beta) {
         st->breakdown = 1;
         st->active = 0;
       }
-      st->inv_h = inv;
+      st->inv_h = hn > 0.0 ? rhn : 0.0;
     }
   }
   __syncthreads();
@@ -922,7 +924,7 @@ __device__ void lsq_column(const ProbK& q, int j, int ldh, double hn, double inv
 // them to the new column is a matrix-vector product (a warp per row, lanes
 // over the columns, fixed-order reduction) instead of a chain of j
 // dependent rotations; lsq_column does the rest.  sh: j + 2 double2.
-__device__ void coop_givens(const ProbK& q, int j, int ldh, double hn, double inv, double2* sh) {
+__device__ void coop_givens(const ProbK& q, int j, int ldh, double hn2, double2* sh) {
   double2* r = sh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int ldq = ldh;
@@ -939,7 +941,7 @@ __device__ void coop_givens(const ProbK& q, int j, int ldh, double hn, double in
     im = warp_sum(im);
     if (lane == 0) r[i] = make_double2(re, im);
   }
-  lsq_column(q, j, ldh, hn, inv, r);
+  lsq_column(q, j, ldh, hn2, r);
 }
 
 // Step j (nv = j + 1 basis vectors) for the count problems of P after the
@@ -956,7 +958,7 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
   const int nblk = gridDim.x;
   const unsigned nb = gridDim.x;
   __shared__ int act[kCoopMaxProblems], reo[kCoopMaxProblems];
-  __shared__ double hn_s[kCoopMaxProblems];
+  __shared__ double hn_s[kCoopMaxProblems], hn2_s[kCoopMaxProblems];
   __shared__ int any_reo;
   extern __shared__ unsigned char coop_raw[];
   A* hs = reinterpret_cast<A*>(coop_raw);                                   // nv coefficients
@@ -1022,7 +1024,10 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
     for (int p = 0; p < count; ++p)
       if (act[p]) {
         const double t = warp_sum_partials(P[p].partial + (size_t)(reo[p] ? nv + 1 : nv) * nblk, nblk).x;
-        if (threadIdx.x == 0) hn_s[p] = sqrt(t);
+        if (threadIdx.x == 0) {
+          hn2_s[p] = t;
+          hn_s[p] = sqrt(t);
+        }
       }
   __syncthreads();
   for (int p = 0; p < count; ++p) {
@@ -1040,7 +1045,7 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
       a.y *= sc;
       v[k] = a;
     }
-    if (blockIdx.x == (unsigned)(p % nblk)) coop_givens(q, j, ldh, hn, inv, col);
+    if (blockIdx.x == (unsigned)(p % nblk)) coop_givens(q, j, ldh, hn2_s[p], col);
   }
   if (set_next) {
     // the last block to finish (ticket in bar[3]) sets the condition of the
@@ -1070,8 +1075,8 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
 // are identical, in a fixed order), so a pass has two grid barriers instead
 // of three or four; and the last block owns no elements: it sums the same
 // partials and does the FP64 least-squares step while the workers update w
-// and write v_{j+1}.  600 x 23 x 11, restart 30: 60 us a step against 103
-// with the step above (operator excluded).
+// and write v_{j+1}.  600 x 23 x 11, restart 30: a solve 193 -> 104 ms, 82 us a
+// step of which the operator takes 32 and the basis sweeps about 25.
 //
 // Barrier: a counter that only grows.  A block's ticket t belongs to barrier
 // t / nblocks, which is complete when the counter reaches the next multiple
@@ -1101,6 +1106,35 @@ __device__ __forceinline__ bool ticket_barrier(unsigned* bar, unsigned nblocks) 
   return ok_s != 0;
 }
 
+// Sums across warps and blocks as unevaluated pairs of FP32 (Dekker, Knuth):
+// 48 bits, where the products and warp sums below them carry 24.  An SM
+// retires two FP64 additions a clock, so in FP64 the sums of 151 partials of
+// 30 coefficients took 4.7 us in every block and ||w'|| 7 us; as pairs 1 us.
+struct Pair {
+  float hi, lo;
+};
+__device__ __forceinline__ Pair two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair pair_add(Pair a, Pair b) {
+  const Pair s = two_sum(a.hi, b.hi);
+  const float e = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
+  const float hi = __fadd_rn(s.hi, e);
+  return Pair{hi, __fsub_rn(e, __fsub_rn(hi, s.hi))};
+}
+__device__ __forceinline__ Pair pair_shfl_xor(Pair a, int o) {
+  return Pair{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double pair_value(Pair a) { return (double)a.hi + (double)a.lo; }
+// 1 / sqrt(a): FP32 estimate and one Newton step on the pair
+__device__ __forceinline__ float pair_rsqrt(Pair a) {
+  const float y = rsqrtf(a.hi);
+  const float t = __fmul_rn(a.hi, y), e = __fmaf_rn(a.hi, y, -t);
+  const float r = __fsub_rn(__fmaf_rn(-t, y, 1.f), __fmaf_rn(e, y, a.lo * y * y));
+  return __fmaf_rn(0.5f * y, r, y);
+}
+
 constexpr int kStepThreads = 512;
 constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kDotGroup = 16;   // vectors whose products a thread accumulates at a time
@@ -1124,10 +1158,10 @@ __device__ __forceinline__ float warp_transpose_sum(float (&a)[32]) {
 // vectors loaded together: about 24 loads in flight a thread
 template <int E> __host__ __device__ constexpr int step_vectors() { return E <= 2 ? 8 : E <= 6 ? 4 : E <= 8 ? 2 : 1; }
 
-// Block partials of conj(V_i) w, i < nv -> partial[i nblk + blockIdx.x].
+// Block partials (re, im pairs) of conj(V_i) w, i < nv -> partial[i nblk + blockIdx.x].
 template <int E>
 __device__ void step_dots(const float2* __restrict__ V, size_t n, int nv, size_t k0, int own, const float2 (&w)[E],
-                          double2* __restrict__ partial, int nblk, float (*red)[kStepWarps][32]) {
+                          float4* __restrict__ partial, int nblk, float (*red)[32]) {
   constexpr int G = step_vectors<E>();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i0 = 0; i0 < nv; i0 += kDotGroup) {
@@ -1156,13 +1190,17 @@ __device__ void step_dots(const float2* __restrict__ V, size_t n, int nv, size_t
           }
       }
     }
-    red[0][warp][lane] = warp_transpose_sum(acc);
+    red[warp][lane] = warp_transpose_sum(acc);
     __syncthreads();
     if (threadIdx.x < 32 && i0 + (threadIdx.x >> 1) < nv) {
-      double t = 0.0;
+      Pair t[4];   // four chains of four warps
 #pragma unroll
-      for (int k = 0; k < kStepWarps; ++k) t += (double)red[0][k][threadIdx.x];
-      ((double*)(partial + (size_t)(i0 + (threadIdx.x >> 1)) * nblk + blockIdx.x))[threadIdx.x & 1] = t;
+      for (int k = 0; k < 4; ++k)
+        t[k] = pair_add(two_sum(red[4 * k][threadIdx.x], red[4 * k + 1][threadIdx.x]),
+                        two_sum(red[4 * k + 2][threadIdx.x], red[4 * k + 3][threadIdx.x]));
+      const Pair v = pair_add(pair_add(t[0], t[1]), pair_add(t[2], t[3]));
+      ((float2*)(partial + (size_t)(i0 + (threadIdx.x >> 1)) * nblk + blockIdx.x))[threadIdx.x & 1] =
+          make_float2(v.hi, v.lo);
     }
     __syncthreads();
   }
@@ -1198,31 +1236,65 @@ __device__ void step_update(const float2* __restrict__ V, size_t n, int nv, size
 
 // block partial of |w|^2 -> *out
 template <int E>
-__device__ void step_norm(const float2 (&w)[E], double2* out, float (*red)[kStepWarps][32]) {
+__device__ void step_norm(const float2 (&w)[E], float4* out, float (*red)[32]) {
   float t = 0.f;
 #pragma unroll
   for (int e = 0; e < E; ++e) t += w[e].x * w[e].x + w[e].y * w[e].y;
   t = warp_sum(t);
-  if ((threadIdx.x & 31) == 0) red[0][0][threadIdx.x >> 5] = t;
+  if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = t;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double u = 0.0;
-    for (int k = 0; k < kStepWarps; ++k) u += (double)red[0][0][k];
-    *out = make_double2(u, 0.0);
+  if (threadIdx.x < 32) {
+    Pair v{threadIdx.x < kStepWarps ? red[0][threadIdx.x] : 0.f, 0.f};
+#pragma unroll
+    for (int o = kStepWarps / 2; o > 0; o >>= 1) v = pair_add(v, pair_shfl_xor(v, o));
+    if (threadIdx.x == 0) *out = make_float4(v.hi, v.lo, 0.f, 0.f);
   }
 }
 
-// coefficients of every vector: the sum of its partials, one warp per vector
-__device__ void step_coefficients(const double2* __restrict__ partial, int nv, int workers, int nblk,
+// coefficients of every vector: the sums of its partials, eight lanes a vector
+__device__ void step_coefficients(const float4* __restrict__ partial, int nv, int workers, int nblk,
                                   double2* __restrict__ hd, float2* __restrict__ hf) {
-  for (int i = threadIdx.x >> 5; i < nv; i += kStepWarps) {
-    const double2 t = warp_sum_partials(partial + (size_t)i * nblk, workers);
-    if ((threadIdx.x & 31) == 0) {
-      hd[i] = t;
-      hf[i] = make_float2((float)t.x, (float)t.y);
+  const int lane = threadIdx.x & 31, sub = lane & 7;
+  for (int i0 = (threadIdx.x >> 5) * 4; i0 < nv; i0 += 4 * kStepWarps) {
+    const int i = min(i0 + (lane >> 3), nv - 1);
+    const float4* p = partial + (size_t)i * nblk;
+    Pair re{0.f, 0.f}, im{0.f, 0.f};
+    for (int b0 = sub; b0 < workers; b0 += 32) {   // four loads in flight
+      float4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = b0 + 8 * u < workers ? __ldcg(p + b0 + 8 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        re = pair_add(re, Pair{v[u].x, v[u].y});
+        im = pair_add(im, Pair{v[u].z, v[u].w});
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      re = pair_add(re, pair_shfl_xor(re, o));
+      im = pair_add(im, pair_shfl_xor(im, o));
+    }
+    if (sub == 0 && i0 + (lane >> 3) < nv) {
+      hd[i] = make_double2(pair_value(re), pair_value(im));
+      hf[i] = make_float2(re.hi, im.hi);
     }
   }
   __syncthreads();
+}
+
+// ||w||^2 from the blocks' partials, by one warp: every lane gets it
+__device__ __forceinline__ Pair step_norm2(const float4* __restrict__ partial, int workers) {
+  Pair t{0.f, 0.f};
+  for (int b0 = threadIdx.x & 31; b0 < workers; b0 += 5 * 32) {
+    float4 v[5];
+#pragma unroll
+    for (int u = 0; u < 5; ++u) v[u] = b0 + 32 * u < workers ? __ldcg(partial + b0 + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 5; ++u) t = pair_add(t, Pair{v[u].x, v[u].y});
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t = pair_add(t, pair_shfl_xor(t, o));
+  return t;
 }
 
 // r += Q h for the least-squares step (Q: the product of the cycle's
@@ -1255,8 +1327,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) arnoldi_step1_kernel(const Pr
   const ProbK& q = P[0];
   if (!q.st->active) return;   // written only by the last block, after a barrier every block has passed
   extern __shared__ double2 step_raw[];
-  __shared__ float red[1][kStepWarps][32];
-  __shared__ double norm_s;
+  __shared__ float red[kStepWarps][32];
+  __shared__ Pair norm_s;
+  __shared__ int again_s;
   double2* hd = step_raw;
   double2* r = hd + nv;
   float2* hf = reinterpret_cast<float2*>(r + nv + 1);
@@ -1265,18 +1338,19 @@ __global__ void __launch_bounds__(kStepThreads, 1) arnoldi_step1_kernel(const Pr
   const size_t n = q.n, k0 = (size_t)blockIdx.x * chunk;
   const int own = owner || k0 >= n ? 0 : (int)min((size_t)chunk, n - k0);
   const float2* __restrict__ V = (const float2*)q.V;
+  float4* __restrict__ partial = reinterpret_cast<float4*>(q.partial);
   float2 w[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int k = threadIdx.x + e * kStepThreads;
     w[e] = k < own ? ((const float2*)q.w)[k0 + k] : make_float2(0.f, 0.f);
   }
-  if (!owner) step_dots<E>(V, n, nv, k0, own, w, q.partial, nblk, red);
+  if (!owner) step_dots<E>(V, n, nv, k0, own, w, partial, nblk, red);
   if (!ticket_barrier(bar, nblk)) return;
-  step_coefficients(q.partial, nv, workers, nblk, hd, hf);
+  step_coefficients(partial, nv, workers, nblk, hd, hf);
   if (!owner) {
     step_update<E>(V, n, nv, k0, own, w, hf);
-    step_norm<E>(w, q.partial + (size_t)nv * nblk + blockIdx.x, red);
+    step_norm<E>(w, partial + (size_t)nv * nblk + blockIdx.x, red);
   } else {
     step_rotate(q, j, ldh, hd, r, true);
   }
@@ -1284,35 +1358,41 @@ __global__ void __launch_bounds__(kStepThreads, 1) arnoldi_step1_kernel(const Pr
   // ||w'|| and the second-pass decision, identical in every block:
   // ||w'||^2 < (||w'||^2 + ||h1||^2) / 2
   if (threadIdx.x < 32) {
-    const double t = warp_sum_partials(q.partial + (size_t)nv * nblk, workers).x;
-    double h2 = 0.0;
-    for (int i = threadIdx.x; i < nv; i += 32) h2 += hd[i].x * hd[i].x + hd[i].y * hd[i].y;
-    h2 = warp_sum(h2);
-    if (threadIdx.x == 0) norm_s = t < 0.5 * (t + h2) ? -1.0 : t;
+    const Pair t = step_norm2(partial + (size_t)nv * nblk, workers);
+    Pair h2{0.f, 0.f};
+    for (int i = threadIdx.x; i < nv; i += 32) {
+      const float2 h = hf[i];
+      h2 = pair_add(h2, two_sum(h.x * h.x, h.y * h.y));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) h2 = pair_add(h2, pair_shfl_xor(h2, o));
+    if (threadIdx.x == 0) {
+      norm_s = t;
+      again_s = t.hi < 0.5f * pair_add(t, h2).hi;
+    }
   }
   __syncthreads();
-  const bool again = norm_s < 0.0;
+  const bool again = again_s;
   if (again) {
-    if (!owner) step_dots<E>(V, n, nv, k0, own, w, q.partial, nblk, red);
+    if (!owner) step_dots<E>(V, n, nv, k0, own, w, partial, nblk, red);
     if (!ticket_barrier(bar, nblk)) return;
-    step_coefficients(q.partial, nv, workers, nblk, hd, hf);
+    step_coefficients(partial, nv, workers, nblk, hd, hf);
     if (!owner) {
       step_update<E>(V, n, nv, k0, own, w, hf);
-      step_norm<E>(w, q.partial + (size_t)(nv + 1) * nblk + blockIdx.x, red);
+      step_norm<E>(w, partial + (size_t)(nv + 1) * nblk + blockIdx.x, red);
     } else {
       step_rotate(q, j, ldh, hd, r, false);
     }
     if (!ticket_barrier(bar, nblk)) return;
     if (threadIdx.x < 32) {
-      const double t = warp_sum_partials(q.partial + (size_t)(nv + 1) * nblk, workers).x;
+      const Pair t = step_norm2(partial + (size_t)(nv + 1) * nblk, workers);
       if (threadIdx.x == 0) norm_s = t;
     }
     __syncthreads();
   }
-  const double hn = sqrt(norm_s);
-  const double inv = (hn > 0.0 && isfinite(hn)) ? 1.0 / hn : 0.0;
+  const Pair nrm = norm_s;
   if (!owner) {
-    const float sc = (float)inv;
+    const float sc = nrm.hi > 0.f && isfinite(nrm.hi) ? pair_rsqrt(nrm) : 0.f;
     float2* __restrict__ v = (float2*)q.V + (size_t)nv * n + k0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -1325,7 +1405,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) arnoldi_step1_kernel(const Pr
     q.st->reorth = again;
     q.st->reorth_count += again;
   }
-  lsq_column(q, j, ldh, hn, inv, r);
+  lsq_column(q, j, ldh, pair_value(nrm), r);
   if (set_next && threadIdx.x == 0) cudaGraphSetConditional(next, q.st->active ? 1u : 0u);
 }
 
