@@ -26,6 +26,7 @@
 //   once from HBM), then z = inverse FFT / nx.  The vectors' planar layout
 //   [p][z][y][x] is already the (3B) x nx matrix the transforms need.
 #include <cuda_fp16.h>
+#include <cuda_pipeline.h>
 #include <math.h>
 #include <stdio.h>
 
@@ -40,7 +41,7 @@ struct vie_circulant {
   int gen = 0;                 // contrast generation the factors were built from
   int nx = 0, ny = 0, nz = 0, B = 0, R = 0, nb = 32;
   float2* W = nullptr;         // nx x R x R: LU factors (unit L below, U on and above the diagonal)
-  __half2* W16 = nullptr;      // the same in complex half precision (VIE_CIRC_FP16_FACTORS; W is then freed)
+  __half2* W16 = nullptr;      // the same in complex half precision, as tiles (VIE_CIRC_FP16_FACTORS; W is then freed)
   bool fp16 = false;
   int* perm = nullptr;         // nx x R: row r of P b is b[perm[r]]
   float2* vh = nullptr;        // nx x R scratch (row-major [w][r])
@@ -507,26 +508,22 @@ __device__ __forceinline__ float2 cdiv(float2 a, float2 b) {
   return make_float2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
 
-__device__ __forceinline__ float2 ld_factor(const float2* p) { return *p; }
-__device__ __forceinline__ float2 ld_factor(const __half2* p) { return __half22float2(*p); }
-
 // Streamer part of the pipelined substitution: 224 threads (warps 1-7),
 // seven per row of a 32-row block row.  Thread (row, sub) sums
-// A[j0 + row][t] x[t] over t = c0 + sub + 7 u < c1 with 16 (complex64) or 32
-// (complex half) loads in flight and leaves the sum in red[row][sub].
-template <typename T>
-__device__ __forceinline__ void stream_partial(const T* __restrict__ A, int R, int j0, int nr, int c0, int c1,
+// A[j0 + row][t] x[t] over t = c0 + sub + 7 u < c1 with 16 loads in flight and
+// leaves the sum in red[row][sub].
+__device__ __forceinline__ void stream_partial(const float2* __restrict__ A, int R, int j0, int nr, int c0, int c1,
                                                const float2* __restrict__ x, float2 (*red)[8], int st) {
   const int row = st / 7, sub = st - row * 7;
   float sx = 0.f, sy = 0.f;
   if (row < nr) {
-    constexpr int U = sizeof(T) == 4 ? 32 : 16;
-    const T* rp = A + (size_t)(j0 + row) * R;
+    constexpr int U = 16;
+    const float2* rp = A + (size_t)(j0 + row) * R;
     int t = c0 + sub;
     for (; t + 7 * (U - 1) < c1; t += 7 * U) {
       float2 l[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) l[u] = ld_factor(rp + t + 7 * u);
+      for (int u = 0; u < U; ++u) l[u] = rp[t + 7 * u];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const float2 xt = x[t + 7 * u];
@@ -535,7 +532,7 @@ __device__ __forceinline__ void stream_partial(const T* __restrict__ A, int R, i
       }
     }
     for (; t < c1; t += 7) {
-      const float2 l = ld_factor(rp + t), xt = x[t];
+      const float2 l = rp[t], xt = x[t];
       sx += l.x * xt.x - l.y * xt.y;
       sy += l.x * xt.y + l.y * xt.x;
     }
@@ -550,14 +547,13 @@ __device__ __forceinline__ void stream_partial(const T* __restrict__ A, int R, i
 // that is already final and prefetch block k+1's diagonal block and its
 // coupling block into the other half of double-buffered shared memory.  One
 // barrier per block.  256 threads.
-template <typename T>
-__global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict__ W, const int* __restrict__ perm,
+__global__ void __launch_bounds__(256, 4) circ_solve_kernel(const float2* __restrict__ W, const int* __restrict__ perm,
                                                          float2* __restrict__ vh, int R) {
   extern __shared__ float2 x[];
   __shared__ float2 D[2][32][33];   // diagonal block
   __shared__ float2 E[2][32][33];   // coupling to the previously solved block
   __shared__ float2 red[2][32][8];  // streamed partial sums, 7 per row
-  const T* A = W + (size_t)blockIdx.x * R * R;
+  const float2* A = W + (size_t)blockIdx.x * R * R;
   const int* pm = perm + (size_t)blockIdx.x * R;
   float2* b = vh + (size_t)blockIdx.x * R;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, st = tid - 32;
@@ -569,7 +565,7 @@ __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict_
     const int nr = nrows(0);
     for (int e = tid; e < 32 * 32; e += blockDim.x) {
       const int a = e >> 5, t = e & 31;
-      D[0][a][t] = (a < nr && t < nr) ? ld_factor(A + (size_t)a * R + t) : make_float2(0.f, 0.f);
+      D[0][a][t] = (a < nr && t < nr) ? A[(size_t)a * R + t] : make_float2(0.f, 0.f);
       if (t < 8) red[0][a][t] = make_float2(0.f, 0.f);
     }
   }
@@ -595,8 +591,8 @@ __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict_
       for (int e = st; e < 32 * 32; e += blockDim.x - 32) {
         const int a = e >> 5, t = e & 31;
         const bool in = a < nr1;
-        D[nxt][a][t] = (in && t < nr1) ? ld_factor(A + (size_t)(j0 + a) * R + j0 + t) : make_float2(0.f, 0.f);
-        E[nxt][a][t] = in ? ld_factor(A + (size_t)(j0 + a) * R + i0 + t) : make_float2(0.f, 0.f);
+        D[nxt][a][t] = (in && t < nr1) ? A[(size_t)(j0 + a) * R + j0 + t] : make_float2(0.f, 0.f);
+        E[nxt][a][t] = in ? A[(size_t)(j0 + a) * R + i0 + t] : make_float2(0.f, 0.f);
       }
     }
     __syncthreads();
@@ -606,7 +602,7 @@ __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict_
     const int kl = nblk - 1, i0 = 32 * kl, nr = nrows(kl);
     for (int e = tid; e < 32 * 32; e += blockDim.x) {
       const int a = e >> 5, t = e & 31;
-      D[0][a][t] = (a < nr && t < nr) ? ld_factor(A + (size_t)(i0 + a) * R + i0 + t) : make_float2(0.f, 0.f);
+      D[0][a][t] = (a < nr && t < nr) ? A[(size_t)(i0 + a) * R + i0 + t] : make_float2(0.f, 0.f);
       if (t < 8) red[0][a][t] = make_float2(0.f, 0.f);
     }
   }
@@ -635,8 +631,8 @@ __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict_
       stream_partial(A, R, j0, 32, i1, R, x, red[nxt], st);
       for (int e = st; e < 32 * 32; e += blockDim.x - 32) {
         const int a = e >> 5, t = e & 31;
-        D[nxt][a][t] = ld_factor(A + (size_t)(j0 + a) * R + j0 + t);
-        E[nxt][a][t] = t < nr ? ld_factor(A + (size_t)(j0 + a) * R + i0 + t) : make_float2(0.f, 0.f);
+        D[nxt][a][t] = A[(size_t)(j0 + a) * R + j0 + t];
+        E[nxt][a][t] = t < nr ? A[(size_t)(j0 + a) * R + i0 + t] : make_float2(0.f, 0.f);
       }
     }
     __syncthreads();
@@ -644,9 +640,161 @@ __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const T* __restrict_
   for (int r = tid; r < R; r += blockDim.x) b[r] = x[r];
 }
 
-__global__ void to_half_kernel(const float2* __restrict__ a, __half2* __restrict__ b, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    b[i] = __float22half2_rn(a[i]);
+// ---------------------------------------------------------------------------
+// complex-half factors: 32 x 32 tiles in the order the substitutions read them
+// ---------------------------------------------------------------------------
+// Of each matrix (nb block rows): forward, block row k = 0 .. nb - 1: L tiles
+// (k, 0) .. (k, k - 1), then the diagonal tile; backward, k = nb - 1 .. 0: U
+// tiles (k, k + 1) .. (k, nb - 1), then the diagonal tile again.  One linear
+// stream of nb (nb + 1) tiles of 4 KB per frequency, which is what lets the
+// substitution keep its loads 16 bytes wide and far ahead.  Off-diagonal tiles
+// are row-major; diagonal ones column-major (the solve walks columns, a lane
+// per row), with the identity beyond row R.
+constexpr int kTile = 32;
+constexpr int kTileElems = kTile * kTile;
+
+__global__ void __launch_bounds__(256) to_tiles_kernel(const float2* __restrict__ W, __half2* __restrict__ F, int R,
+                                                       int nb) {
+  const float2* A = W + (size_t)blockIdx.y * R * R;
+  const int t = blockIdx.x, half = nb * (nb + 1) / 2;
+  __half2* out = F + ((size_t)blockIdx.y * 2 * half + t) * kTileElems;
+  // block row and position of tile t of a direction: rows have 1, 2, .. nb tiles
+  const int u = t < half ? t : t - half;
+  int k = (int)((sqrtf(8.f * u + 1.f) - 1.f) * 0.5f);
+  while (k * (k + 1) / 2 > u) --k;
+  while ((k + 1) * (k + 2) / 2 <= u) ++k;
+  const int i = u - k * (k + 1) / 2;               // i == k: the diagonal tile
+  const int row = t < half ? k : nb - 1 - k;
+  const int col = i == k ? row : (t < half ? i : row + 1 + i);
+  __shared__ __half2 D[kTile][kTile + 1];
+  for (int e = threadIdx.x; e < kTileElems; e += 256) {
+    const int r = e >> 5, c = e & 31, gr = row * kTile + r, gc = col * kTile + c;
+    float2 v = make_float2(i == k && gr == gc ? 1.f : 0.f, 0.f);
+    if (gr < R && gc < R) v = A[(size_t)gr * R + gc];
+    if (i == k) D[c][r] = __float22half2_rn(v);
+    else out[e] = __float22half2_rn(v);
+  }
+  if (i != k) return;
+  __syncthreads();
+  for (int e = threadIdx.x; e < kTileElems; e += 256) out[e] = D[e >> 5][e & 31];
+}
+
+// x = P b, then L y = x and U z = y from the tile stream, one CTA per
+// frequency.  HBM-bound: the factors are read once.  A stage is up to four
+// tiles of one block row (16 KB); two stages are in flight (asynchronous
+// copies) while one is used, 32 KB a CTA, four CTAs an SM.  Warp w sums rows
+// 4 w .. 4 w + 3 of a tile, a lane per column; at the end of a block row the
+// sums meet in shared memory and warp 0 solves the diagonal tile.  The rows
+// used to be read by seven threads each, 4 bytes at a time: 599 us for 396
+// frequencies of 1080 unknowns.
+constexpr int kStageTiles = 4;
+constexpr int kSolveStages = 3;
+
+struct TileRow {   // position in the stream: direction, block row, next tile of the row
+  int dir, k, i;
+  __device__ __forceinline__ int count() const { return min(kStageTiles, k + 1 - i); }
+  __device__ __forceinline__ void next(int nb) {
+    i += kStageTiles;
+    if (i > k) {
+      i = 0;
+      if (++k == nb) { k = 0; ++dir; }
+    }
+  }
+};
+
+__global__ void __launch_bounds__(256, 4) circ_solve_tiles_kernel(const __half2* __restrict__ F,
+                                                                  const int* __restrict__ perm,
+                                                                  float2* __restrict__ vh, int R, int nb) {
+  extern __shared__ __align__(16) unsigned char circ_smem[];
+  __half2* ring = reinterpret_cast<__half2*>(circ_smem);                                  // [stage][tile][1024]
+  float2* x = reinterpret_cast<float2*>(ring + kSolveStages * kStageTiles * kTileElems);  // nb kTile
+  __shared__ float psum[2 * kTile];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const __half2* src = F + (size_t)blockIdx.x * nb * (nb + 1) * kTileElems;
+  const int* pm = perm + (size_t)blockIdx.x * R;
+  float2* b = vh + (size_t)blockIdx.x * R;
+  TileRow ahead{0, 0, 0}, at{0, 0, 0};
+  auto issue = [&](int slot) {   // the next stage's copies into a slot (an empty group past the end)
+    if (ahead.dir < 2) {
+      const int n = ahead.count();
+      for (int t = 0; t < n; ++t)
+        __pipeline_memcpy_async(ring + (slot * kStageTiles + t) * kTileElems + tid * 4,
+                                src + (size_t)t * kTileElems + tid * 4, 16);
+      src += (size_t)n * kTileElems;
+      ahead.next(nb);
+    }
+    __pipeline_commit();
+  };
+  issue(0);
+  issue(1);
+  for (int r = tid; r < nb * kTile; r += 256) x[r] = r < R ? b[pm[r]] : make_float2(0.f, 0.f);
+  float acc[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) acc[u] = 0.f;
+  for (int slot = 0; at.dir < 2; slot = slot == kSolveStages - 1 ? 0 : slot + 1) {
+    __pipeline_wait_prior(kSolveStages - 2);
+    __syncthreads();   // the stage has landed for every thread; the slot of the one before is free
+    issue(slot == 0 ? kSolveStages - 1 : slot - 1);
+    const int n = at.count();
+    const bool last = at.i + n > at.k;                      // the row's diagonal tile is the stage's last
+    const int row = at.dir == 0 ? at.k : nb - 1 - at.k;
+    const __half2* tile = ring + slot * kStageTiles * kTileElems;
+    for (int t = 0; t < n - (last ? 1 : 0); ++t) {
+      const int col = at.dir == 0 ? at.i + t : row + 1 + at.i + t;
+      const float2 xt = x[col * kTile + lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float2 l = __half22float2(tile[t * kTileElems + (4 * warp + u) * kTile + lane]);
+        acc[2 * u] += l.x * xt.x - l.y * xt.y;
+        acc[2 * u + 1] += l.x * xt.y + l.y * xt.x;
+      }
+    }
+    if (last) {
+      // eight sums a lane over the warp: after three exchanges a lane holds one
+#pragma unroll
+      for (int o = 16, k = 4; k >= 1; o >>= 1, k >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int u = 0; u < k; ++u) {
+          const float keep = up ? acc[u + k] : acc[u], give = up ? acc[u] : acc[u + k];
+          acc[u] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      }
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+      if ((lane & 3) == 0) psum[8 * warp + (lane >> 2)] = acc[0];   // lane bits 4, 3, 2: the value's index
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc[u] = 0.f;
+      __syncthreads();
+      if (warp == 0) {
+        const __half2* D = tile + (n - 1) * kTileElems;     // column-major
+        float2 xi = x[row * kTile + lane];
+        xi.x -= psum[2 * lane];
+        xi.y -= psum[2 * lane + 1];
+        if (at.dir == 0) {
+#pragma unroll 8
+          for (int t = 0; t < kTile - 1; ++t) {
+            const float2 l = __half22float2(D[t * kTile + lane]);
+            const float2 xt = make_float2(__shfl_sync(0xffffffffu, xi.x, t), __shfl_sync(0xffffffffu, xi.y, t));
+            if (lane > t) xi = csub_mul(xi, l, xt);
+          }
+        } else {
+          const float2 inv = cdiv(make_float2(1.f, 0.f), __half22float2(D[lane * kTile + lane]));
+#pragma unroll 8
+          for (int t = kTile - 1; t >= 0; --t) {
+            const float2 l = __half22float2(D[t * kTile + lane]);
+            if (lane == t) xi = cmul(xi, inv);
+            const float2 xt = make_float2(__shfl_sync(0xffffffffu, xi.x, t), __shfl_sync(0xffffffffu, xi.y, t));
+            if (lane < t) xi = csub_mul(xi, l, xt);
+          }
+        }
+        x[row * kTile + lane] = xi;
+      }
+    }
+    at.next(nb);
+  }
+  __syncthreads();
+  for (int r = tid; r < R; r += 256) b[r] = x[r];
 }
 
 __global__ void to_c64_kernel(const double2* __restrict__ a, float2* __restrict__ b, size_t n) {
@@ -794,8 +942,14 @@ vie_status circulant_apply(vie_circulant* c, int dtype, const void* v, void* z, 
   // V_hat[w][r] = sum_x exp(-2 pi i w x / nx) v[r][x]
   lines_fft_kernel<false><<<(R + kLines - 1) / kLines, 256, fft_smem, s>>>(vin, c->vh, R, nx, c->rd, c->tw);
   VIE_LAUNCH_CHECK();
-  if (c->fp16) circ_solve_kernel<__half2><<<nx, 256, (size_t)R * sizeof(float2), s>>>(c->W16, c->perm, c->vh, R);
-  else circ_solve_kernel<float2><<<nx, 256, (size_t)R * sizeof(float2), s>>>(c->W, c->perm, c->vh, R);
+  if (c->fp16) {
+    const int nb = (R + kTile - 1) / kTile;
+    const size_t smem = (size_t)kSolveStages * kStageTiles * kTileElems * sizeof(__half2) + (size_t)nb * kTile * sizeof(float2);
+    VIE_CUDA_TRY(cudaFuncSetAttribute(circ_solve_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    circ_solve_tiles_kernel<<<nx, 256, smem, s>>>(c->W16, c->perm, c->vh, R, nb);
+  } else {
+    circ_solve_kernel<<<nx, 256, (size_t)R * sizeof(float2), s>>>(c->W, c->perm, c->vh, R);
+  }
   VIE_LAUNCH_CHECK();
   // z[r][x] = (1/nx) sum_w exp(+2 pi i w x / nx) Z_hat[w][r]
   lines_fft_kernel<true><<<(R + kLines - 1) / kLines, 256, fft_smem, s>>>(c->vh, zout, R, nx, c->rd, c->tw);
@@ -858,10 +1012,10 @@ vie_status vie_circulant_create(vie_plan* plan, int flags, vie_circulant** out, 
   vie_status st = circ_build(c, (cudaStream_t)stream, (size_t)smem_optin);
   if (st == VIE_OK && (flags & VIE_CIRC_FP16_FACTORS)) {
     // keep only a complex-half copy of the factors
-    const size_t ne = (size_t)c->nx * c->R * c->R;
-    cudaError_t e = cudaMalloc((void**)&c->W16, ne * sizeof(__half2));
+    const int nb = (c->R + kTile - 1) / kTile, tiles = nb * (nb + 1);
+    cudaError_t e = cudaMalloc((void**)&c->W16, (size_t)c->nx * tiles * kTileElems * sizeof(__half2));
     if (e == cudaSuccess) {
-      to_half_kernel<<<blocks_for(ne), 256, 0, (cudaStream_t)stream>>>(c->W, c->W16, ne);
+      to_tiles_kernel<<<dim3((unsigned)tiles, (unsigned)c->nx), 256, 0, (cudaStream_t)stream>>>(c->W, c->W16, c->R, nb);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
@@ -894,8 +1048,10 @@ vie_status vie_circulant_info(const vie_circulant* c, double* build_ms, size_t* 
   clear_error();
   if (!c) { set_error("null argument"); return VIE_ERR_INVALID; }
   if (build_ms) *build_ms = c->build_ms;
+  const size_t nb = (size_t)(c->R + kTile - 1) / kTile;
   if (device_bytes)
-    *device_bytes = (size_t)c->nx * c->R * c->R * (c->fp16 ? sizeof(__half2) : sizeof(float2)) +
+    *device_bytes = (c->fp16 ? (size_t)c->nx * nb * (nb + 1) * kTileElems * sizeof(__half2)
+                             : (size_t)c->nx * c->R * c->R * sizeof(float2)) +
                     (size_t)c->nx * c->R * (sizeof(int) + sizeof(float2)) + (size_t)c->nx * sizeof(float2) +
                     (size_t)2 * c->nx * c->R * sizeof(float2);
   return VIE_OK;
