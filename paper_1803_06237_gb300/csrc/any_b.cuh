@@ -9,7 +9,11 @@
 namespace vie {
 
 // ---------------------------------------------------------------------------
-// pass B, one CTA per kx.  z lines (Mz <= 32) in one thread's registers; y
+// pass B, one CTA per kx.  z lines (Mz <= 32) in registers: half of a z
+// line's inputs are padding and half of its outputs are cropped, so for even
+// Mz the radix-2 step falls apart into two transforms of Mz / 2 points, even
+// and odd frequencies, by two neighbouring lanes (complex64; the half step's
+// twiddles cost FP64, which binds complex128, 5 % more); y
 // lines My = r1 r2 in two in-place stages, n = n2 + r2 n1, ky = k1 + r1 k2.
 // The second forward stage, the spectral product and the first inverse stage
 // need the same (kz, k1) group of r2 values of every component, so one thread
@@ -18,10 +22,24 @@ namespace vie {
 // Place of (c, kz; n1 or k1, n2): (c Mz + kz) py + p2 k1 + n2, p2 = r2 | 1,
 // py = r1 p2: rows of stage items and of fused items fall on distinct banks.
 // ---------------------------------------------------------------------------
+// Sizes known at compile time (the benchmark's 460 x 220 nm strip, 23 x 11
+// voxels in 45 or 48 x 24): the same kernel with its divisions, strides and
+// switches folded.  Zeros: all at run time.
+template <int R1_, int R2_, int MZ_, int NY_, int NZ_, int PY_>
+struct BFix {
+  static constexpr int R1 = R1_, R2 = R2_, MZ = MZ_, NY = NY_, NZ = NZ_, PY = PY_, P2 = R2_ | 1;
+  static constexpr bool on = R1_ > 0;
+};
+typedef BFix<0, 0, 0, 0, 0, 0> BFree;
+
 #define VIE_Z_LENGTHS(X) \
   X(1) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(12) X(15) X(16) X(18) X(20) X(24) X(25) X(27) X(30) X(32)
-template <int TOP, typename F>
+template <int TOP, typename FIX, typename F>
 __device__ __forceinline__ void with_z(int mz, F&& f) {
+  if constexpr (FIX::on) {
+    f(IC<FIX::MZ>{});
+    return;
+  }
   switch (mz) {
 #define VIE_X(a) case a: if constexpr (a <= TOP) f(IC<a>{}); break;
     VIE_Z_LENGTHS(VIE_X)
@@ -42,8 +60,12 @@ struct BAny {
 };
 
 #define VIE_R1(X) X(1) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(12) X(15) X(16)
-template <int TOP, typename F>
+template <int TOP, typename FIX, typename F>
 __device__ __forceinline__ void with_r1(int r, F&& f) {
+  if constexpr (FIX::on) {
+    f(IC<FIX::R1>{});
+    return;
+  }
   switch (r) {
 #define VIE_X(a) case a: if constexpr (a <= TOP) f(IC<a>{}); break;
     VIE_R1(VIE_X)
@@ -53,8 +75,12 @@ __device__ __forceinline__ void with_r1(int r, F&& f) {
 }
 // largest fused radix: the group of nc r2 complex values lives in registers
 template <typename V, int NC> __host__ __device__ constexpr int fused_max() { return sizeof(V) * NC <= 24 ? 10 : 6; }
-template <int TOP, typename F>
+template <int TOP, typename FIX, typename F>
 __device__ __forceinline__ void with_r2(int r, F&& f) {
+  if constexpr (FIX::on) {
+    f(IC<FIX::R2>{});
+    return;
+  }
   switch (r) {
     case 1: f(IC<1>{}); break;
     case 2: f(IC<2>{}); break;
@@ -69,7 +95,19 @@ __device__ __forceinline__ void with_r2(int r, F&& f) {
   }
 }
 
-template <typename V, int NC, bool STAGE, bool SMALL>
+// a[z] times exp(-/+ 2 pi i z / L), z < L / 2 (the odd frequencies' input, or
+// the conjugate on their output)
+template <typename V, bool INV, int L>
+__device__ __forceinline__ void half_twiddle(V (&a)[L / 2]) {
+  typedef typename real_of<V>::type T;
+  static_for<1, L / 2>([&](auto zc) {
+    constexpr int z = decltype(zc)::value;
+    typedef TwConst<L, z> W;
+    a[z] = mul_cs(a[z], (T)W::c, INV ? -(T)W::s : (T)W::s);
+  });
+}
+
+template <typename V, int NC, bool STAGE, bool SMALL, typename FIX>
 __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && NC == 3 ? 3 : 2) : 1) pass_b_any_kernel(
     const __grid_constant__ PassPtrs<V> pp, const V* __restrict__ chat, double kappa, PassBGeom g, BAny q,
     const V* __restrict__ twy) {
@@ -79,10 +117,16 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
   extern __shared__ unsigned char smem_raw[];
   V* S = reinterpret_cast<V*>(smem_raw);
   const int kx = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  const int ny = g.ny, nz = g.nz, Mz = g.Mz, py = q.py;
+  const int ny = FIX::on ? FIX::NY : g.ny, nz = FIX::on ? FIX::NZ : g.nz, Mz = FIX::on ? FIX::MZ : g.Mz;
+  const int r1 = FIX::on ? FIX::R1 : q.r1, r2 = FIX::on ? FIX::R2 : q.r2;
+  const int p2 = FIX::on ? FIX::P2 : q.p2, py = FIX::on ? FIX::PY : q.py;
+  const int My = FIX::on ? FIX::R1 * FIX::R2 : g.My, Ky = FIX::on ? My / 2 + 1 : g.Ky;
+  auto by_ny = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::NY : 1) : div_by(v, q.mny); };
+  auto by_r1 = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::R1 : 1) : div_by(v, q.mr1); };
+  auto by_r2 = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::R2 : 1) : div_by(v, q.mr2); };
   const bool fx = kx > g.Mx - kx;
   const int kxf = fx ? g.Mx - kx : kx;
-  const int cs = g.Kz * g.Ky;
+  const int cs = FIX::on ? (Mz / 2 + 1) * Ky : g.Kz * g.Ky;
   const V* G = pp.ghat[blockIdx.y] + (size_t)kxf * 6 * cs;
   const V* Cc = NC == 6 ? chat + (size_t)kxf * 3 * cs : nullptr;
   pdl_launch_dependents();
@@ -97,41 +141,57 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
   }
   pdl_wait();
   V* slab = pp.work[blockIdx.y] + (size_t)kx * g.NL;
-  with_z<ZTOP>(Mz, [&](auto zc) {
+  with_z<ZTOP, FIX>(Mz, [&](auto zc) {
     constexpr int MZ = decltype(zc)::value;
-    for (int line = tid; line < NC * ny; line += nth) {
-      const int c = div_by(line, q.mny), y = line - c * ny;
-      V a[MZ];
+    if constexpr (MZ % 2 == 0 && sizeof(V) == sizeof(float2)) {
+      constexpr int M = MZ / 2;
+      for (int it = tid; it < 2 * NC * ny; it += nth) {
+        const int line = it >> 1, odd = it & 1;
+        const int c = by_ny(line), y = line - c * ny;
+        V a[M];
 #pragma unroll
-      for (int z = 0; z < MZ; ++z) a[z] = (z < (MZ + 1) / 2 && z < nz) ? slab[(c * nz + z) * ny + y] : zero_c<V>();
-      reg_fft<V, false, MZ, (MZ + 1) / 2>(a, nullptr);
-      V* d = S + c * MZ * py + y + (q.p2 - q.r2) * div_by(y, q.mr2);
+        for (int z = 0; z < M; ++z) a[z] = z < nz ? slab[(c * nz + z) * ny + y] : zero_c<V>();
+        if (odd) half_twiddle<V, false, MZ>(a);
+        reg_fft<V, false, M>(a, nullptr);
+        V* d = S + (c * MZ + odd) * py + y + (p2 - r2) * by_r2(y);
 #pragma unroll
-      for (int kz = 0; kz < MZ; ++kz) d[kz * py] = a[kz];
+        for (int k = 0; k < M; ++k) d[2 * k * py] = a[k];
+      }
+    } else {
+      for (int line = tid; line < NC * ny; line += nth) {
+        const int c = by_ny(line), y = line - c * ny;
+        V a[MZ];
+#pragma unroll
+        for (int z = 0; z < MZ; ++z) a[z] = (z < (MZ + 1) / 2 && z < nz) ? slab[(c * nz + z) * ny + y] : zero_c<V>();
+        reg_fft<V, false, MZ, (MZ + 1) / 2>(a, nullptr);
+        V* d = S + c * MZ * py + y + (p2 - r2) * by_r2(y);
+#pragma unroll
+        for (int kz = 0; kz < MZ; ++kz) d[kz * py] = a[kz];
+      }
     }
   });
   __syncthreads();
-  with_r1<R1TOP>(q.r1, [&](auto rc) {
+  with_r1<R1TOP, FIX>(r1, [&](auto rc) {
     constexpr int R1 = decltype(rc)::value;
-    for (int it = tid; it < NC * Mz * q.r2; it += nth) {
-      const int row = div_by(it, q.mr2), n2 = it - row * q.r2;
+    for (int it = tid; it < NC * Mz * r2; it += nth) {
+      const int row = by_r2(it), n2 = it - row * r2;
       V* d = S + row * py + n2;
       V a[R1];
 #pragma unroll
       for (int n1 = 0; n1 < R1; ++n1)
-        a[n1] = (n1 < (R1 + 1) / 2 && n2 + q.r2 * n1 < ny) ? d[n1 * q.p2] : zero_c<V>();
+        a[n1] = (n1 < (R1 + 1) / 2 && n2 + r2 * n1 < ny) ? d[n1 * p2] : zero_c<V>();
       reg_fft<V, false, R1, (R1 + 1) / 2>(a, nullptr);
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) d[k1 * q.p2] = a[k1];
+      for (int k1 = 0; k1 < R1; ++k1) d[k1 * p2] = a[k1];
     }
   });
   if (STAGE) __pipeline_wait_prior(0);
   __syncthreads();
-  with_r2<R2TOP>(q.r2, [&](auto rc) {
+  with_r2<R2TOP, FIX>(r2, [&](auto rc) {
     constexpr int R2 = decltype(rc)::value;
-    for (int it = tid; it < Mz * q.r1; it += nth) {
-      const int kz = div_by(it, q.mr1), k1 = it - kz * q.r1;
-      V* d = S + kz * py + k1 * q.p2;
+    for (int it = tid; it < Mz * r1; it += nth) {
+      const int kz = by_r1(it), k1 = it - kz * r1;
+      V* d = S + kz * py + k1 * p2;
       const int stride = Mz * py;
       V u[NC][R2];
 #pragma unroll
@@ -143,13 +203,13 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
 #pragma unroll
       for (int c = 0; c < NC; ++c) reg_fft<V, false, R2>(u[c], nullptr);
       const bool fz = kz > Mz - kz;
-      const V* Gz = G + (fz ? Mz - kz : kz) * g.Ky;
-      const V* Cz = NC == 6 ? Cc + (fz ? Mz - kz : kz) * g.Ky : nullptr;
+      const V* Gz = G + (fz ? Mz - kz : kz) * Ky;
+      const V* Cz = NC == 6 ? Cc + (fz ? Mz - kz : kz) * Ky : nullptr;
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) {
-        const int ky = k1 + q.r1 * k2;
-        const bool fy = ky > g.My - ky;
-        const int o = fy ? g.My - ky : ky;
+        const int ky = k1 + r1 * k2;
+        const bool fy = ky > My - ky;
+        const int o = fy ? My - ky : ky;
         const V gxx = Gz[o], gyy = Gz[cs + o], gzz = Gz[2 * cs + o];
         V gxy = Gz[3 * cs + o], gxz = Gz[4 * cs + o], gyz = Gz[5 * cs + o];
         if (fx ^ fy) gxy = scale(gxy, (R)-1);
@@ -191,33 +251,63 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
     }
   });
   __syncthreads();
-  with_r1<R1TOP>(q.r1, [&](auto rc) {
+  with_r1<R1TOP, FIX>(r1, [&](auto rc) {
     constexpr int R1 = decltype(rc)::value;
-    for (int it = tid; it < NC * Mz * q.r2; it += nth) {
-      const int row = div_by(it, q.mr2), n2 = it - row * q.r2;
+    for (int it = tid; it < NC * Mz * r2; it += nth) {
+      const int row = by_r2(it), n2 = it - row * r2;
       V* d = S + row * py + n2;
       V a[R1];
 #pragma unroll
-      for (int k1 = 0; k1 < R1; ++k1) a[k1] = d[k1 * q.p2];
+      for (int k1 = 0; k1 < R1; ++k1) a[k1] = d[k1 * p2];
       reg_fft<V, true, R1>(a, nullptr);
 #pragma unroll
       for (int n1 = 0; n1 < (R1 + 1) / 2; ++n1)
-        if (n2 + q.r2 * n1 < ny) d[n1 * q.p2] = a[n1];
+        if (n2 + r2 * n1 < ny) d[n1 * p2] = a[n1];
     }
   });
   __syncthreads();
-  with_z<ZTOP>(Mz, [&](auto zc) {
+  with_z<ZTOP, FIX>(Mz, [&](auto zc) {
     constexpr int MZ = decltype(zc)::value;
-    for (int line = tid; line < NC * ny; line += nth) {
-      const int c = div_by(line, q.mny), y = line - c * ny;
-      const V* d = S + c * MZ * py + y + (q.p2 - q.r2) * div_by(y, q.mr2);
-      V a[MZ];
+    if constexpr (MZ % 2 == 0 && sizeof(V) == sizeof(float2)) {
+      // even and odd frequencies by lanes 2 l, 2 l + 1: x[z] = E[z] + w^-z O[z];
+      // each lane finishes half of the outputs
+      constexpr int M = MZ / 2, H = (M + 1) / 2;
+      const int total = 2 * NC * ny, turns = (total + nth - 1) / nth;
+      for (int turn = 0, it = tid; turn < turns; ++turn, it += nth) {   // every lane takes every turn (shuffles)
+        const bool in = it < total;
+        const int line = in ? it >> 1 : 0, odd = it & 1;
+        const int c = by_ny(line), y = line - c * ny;
+        const V* d = S + (c * MZ + odd) * py + y + (p2 - r2) * by_r2(y);
+        V a[M];
 #pragma unroll
-      for (int kz = 0; kz < MZ; ++kz) a[kz] = d[kz * py];
-      reg_fft<V, true, MZ>(a, nullptr);
+        for (int k = 0; k < M; ++k) a[k] = d[2 * k * py];
+        reg_fft<V, true, M>(a, nullptr);
+        if (odd) half_twiddle<V, true, MZ>(a);
+        V* o = slab + (c * nz) * ny + y;
 #pragma unroll
-      for (int z = 0; z < (MZ + 1) / 2; ++z)
-        if (z < nz) slab[(c * nz + z) * ny + y] = a[z];
+        for (int h = 0; h < H; ++h) {
+          // even lane: z = h (gives E[z'] of the other half), odd lane: z' = h + H
+          V give = odd ? a[h] : (h + H < M ? a[h + H] : zero_c<V>());
+          V got;
+          got.x = __shfl_xor_sync(0xffffffffu, give.x, 1);
+          got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
+          const int z = odd ? h + H : h;
+          const V mine = odd ? (h + H < M ? a[h + H] : zero_c<V>()) : a[h];
+          if (in && z < nz) o[z * ny] = add(mine, got);
+        }
+      }
+    } else {
+      for (int line = tid; line < NC * ny; line += nth) {
+        const int c = by_ny(line), y = line - c * ny;
+        const V* d = S + c * MZ * py + y + (p2 - r2) * by_r2(y);
+        V a[MZ];
+#pragma unroll
+        for (int kz = 0; kz < MZ; ++kz) a[kz] = d[kz * py];
+        reg_fft<V, true, MZ>(a, nullptr);
+#pragma unroll
+        for (int z = 0; z < (MZ + 1) / 2; ++z)
+          if (z < nz) slab[(c * nz + z) * ny + y] = a[z];
+      }
     }
   });
 }
@@ -279,6 +369,12 @@ template <typename V, int NC>
 static vie_status launch_b_any_nc(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* chat, double kappa,
                                   const V* twy, cudaStream_t s, bool* done) {
   *done = false;
+  // small complex128 planes, at most one an SM, or three where one warp holds
+  // all z lines: the generic pass spreads them over more warps (20 x 9 x 6: 44
+  // us an application against 55; 152 x 9 x 14: 156 against 169)
+  if (sizeof(V) == sizeof(double2) && (((long)g.Mx * count <= kSMs && g.My * g.Mz < 500) ||
+                                       (NC * g.ny <= 32 && (long)g.Mx * count <= 3 * kSMs)))
+    return VIE_OK;
   BAny q;
   if (!z_length_any(g.Mz) || !b_any_split<V, NC>(g.ny, g.My, &q)) return VIE_OK;
   const size_t plane = (size_t)NC * g.Mz * q.py * sizeof(V);
@@ -296,14 +392,35 @@ static vie_status launch_b_any_nc(const PassPtrs<V>& pp, int count, const PassBG
   const int threads = ((lines + turns - 1) / turns + 31) / 32 * 32;
   const dim3 grid((unsigned)g.Mx, (unsigned)count);
   const bool small = g.Mz <= 24 && q.r1 <= 10 && q.r2 <= 6;
-  auto run = [&](auto kernel) -> vie_status {
+  auto run = [&](auto kernel, int threads) -> vie_status {
     VIE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    VIE_CUDA_TRY(launch_pdl(kernel, grid, dim3(threads), smem, s, pp, chat, kappa, g, q, twy));
+    VIE_CUDA_TRY(launch_pdl_if(b_starts_early<V>(g, count), kernel, grid, dim3(threads), smem, s, pp, chat, kappa, g, q, twy));
     return VIE_OK;
   };
   vie_status st;
-  if (stage) st = small ? run(pass_b_any_kernel<V, NC, true, true>) : run(pass_b_any_kernel<V, NC, true, false>);
-  else st = small ? run(pass_b_any_kernel<V, NC, false, true>) : run(pass_b_any_kernel<V, NC, false, false>);
+  if constexpr (sizeof(V) == sizeof(float2)) {
+    // the compiled sizes, where they are what was chosen for this plane (the
+    // shared memory above is laid out with q's radices and pitch)
+    auto is = [&](auto fix) {
+      typedef decltype(fix) F;
+      return g.ny == F::NY && g.nz == F::NZ && g.Mz == F::MZ && g.My == F::R1 * F::R2 && q.r1 == F::R1 &&
+             q.r2 == F::R2 && q.p2 == F::P2 && q.py == F::PY && g.Ky == g.My / 2 + 1 && g.Kz == g.Mz / 2 + 1;
+    };
+    typedef BFix<9, 5, 24, 23, 11, 45> F45;
+    typedef BFix<8, 6, 24, 23, 11, 70> F48;
+    if (stage && (is(F45{}) || is(F48{}))) {
+      // five warps for three components: two turns of the fused phase and three
+      // of the first y stage (600 x 23 x 11: 30.7 us an application against
+      // 31.8 with seven, 33.7 with four warps)
+      const int t = NC == 3 ? 160 : threads;
+      st = is(F45{}) ? run(pass_b_any_kernel<V, NC, true, true, F45>, t) : run(pass_b_any_kernel<V, NC, true, true, F48>, t);
+      if (st != VIE_OK) return st;
+      *done = true;
+      return VIE_OK;
+    }
+  }
+  if (stage) st = small ? run(pass_b_any_kernel<V, NC, true, true, BFree>, threads) : run(pass_b_any_kernel<V, NC, true, false, BFree>, threads);
+  else st = small ? run(pass_b_any_kernel<V, NC, false, true, BFree>, threads) : run(pass_b_any_kernel<V, NC, false, false, BFree>, threads);
   if (st != VIE_OK) return st;
   *done = true;
   return VIE_OK;

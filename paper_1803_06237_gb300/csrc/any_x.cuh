@@ -238,7 +238,10 @@ __global__ void __launch_bounds__(x_any_threads<V, TOP>(), 1) pass_c_any_kernel(
 // Split of len into at most three radices (within the small class TOP = 16
 // where possible, then the fewest stages, the smallest largest radix, the
 // smallest sum; the outer radix the largest): false where there is none.
-static bool x_any_split(int len, XAny* g) {
+// small (complex128): the smallest largest radix before the fewest stages, as
+// more butterflies keep the FP64 pipes of more warps busy on short lines (73 x
+// 11 x 9: 65 us an application against 78).
+static bool x_any_split(int len, bool small, XAny* g) {
   long best = -1;
   for (int r1 : kRadices) {
     if (len % r1) continue;
@@ -249,7 +252,7 @@ static bool x_any_split(int len, XAny* g) {
       bool known = false;
       for (int r : kRadices) known |= r == r2;
       if (!known) continue;
-      const long cost = (r1 > 16 ? 1000000L : 0) + (r2 > 1 ? 10000L : 0) + r1 * 100L + r1 + r2 + r3;
+      const long cost = (r1 > 16 ? 1000000L : 0) + (r2 > 1 && !small ? 10000L : 0) + r1 * 100L + r1 + r2 + r3;
       if (best >= 0 && cost >= best) continue;
       best = cost;
       *g = XAny{len, r1, r2, r3, r2 * r3, r3 | 1, 0, 0, 0, div_magic(r2), div_magic(r3), 0};
@@ -311,7 +314,7 @@ vie_status launch_x_any(bool forward, const PassPtrs<V>& pp, int count, int n, i
                         int mode, cudaStream_t s, int gsz, bool* done) {
   *done = false;
   XAny g;
-  if (!x_any_split(len, &g)) return VIE_OK;
+  if (!x_any_split(len, sizeof(V) == sizeof(double2), &g)) return VIE_OK;
   int per = 1;
   const int lpb = x_any_lines(NL, count, (size_t)g.r1 * g.r2 * g.p3 * sizeof(V), &per);
   if (!lpb) return VIE_OK;

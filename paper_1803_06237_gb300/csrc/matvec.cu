@@ -516,10 +516,7 @@ static vie_status dispatch_pass_bz(const PassPtrs<V>& pp, int count, const PassB
 // threads walking their own rows hit distinct banks.
 //   S1: (c, kz) y-lines, pitch PY;  S2: (c, y) z-lines, pitch PZ.
 // ---------------------------------------------------------------------------
-// NY, NZ > 0 fix the cross-section at compile time: the zero padding is not
-// loaded and the cropped outputs are dead code (the first-stage additions of
-// the padding zeros stay: IEEE arithmetic keeps x + 0).
-template <typename V, int MY, int MZ, int NY, int NZ>
+template <typename V, int MY, int MZ>
 __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g,
                                                          const V* __restrict__ twyg, const V* __restrict__ twzg) {
   if (skip_problem(pp)) return;
@@ -535,7 +532,7 @@ __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__
   V* Gs = S2 + 3 * g.ny * PZ;          // folded spectrum chunk of this kx, 6 Kz Ky
   const int kx = blockIdx.x;
   const int tid = threadIdx.x, nth = blockDim.x;
-  const int ny = NY > 0 ? NY : g.ny, nz = NZ > 0 ? NZ : g.nz;
+  const int ny = g.ny, nz = g.nz;
   const bool fx = kx > g.Mx - kx;
   const int kxf = fx ? g.Mx - kx : kx;
   pdl_launch_dependents();
@@ -624,12 +621,11 @@ __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__
   }
 }
 
-// (MY, MZ) pairs with a register-FFT pass B; other sizes use pass_b_kernel.
+// (MY, MZ) pairs with this pass B: at these planes it is up to a tenth faster
+// than the kernel with run-time radices (500 x 24 x 13: 34.6 us an application
+// against 38.8), which serves every other size.
 #define VIE_PASS_B_REG_SIZES(X) \
   X(24, 24) X(45, 24) X(48, 24) X(50, 24) X(30, 24) X(40, 24) X(25, 24) X(45, 25) X(48, 25) X(24, 25)
-// (MY, MZ, NY, NZ) with the cross-section compiled in: the 460 x 220 nm strip
-// at 20 nm (23 x 11 voxels) in its smallest 5-smooth embeddings.
-#define VIE_PASS_B_REG_FIXED(X) X(45, 24, 23, 11) X(48, 24, 23, 11)
 
 bool pass_b_reg_available(int my, int mz) {
 #define VIE_X(a, b) if (my == a && mz == b) return true;
@@ -638,30 +634,30 @@ bool pass_b_reg_available(int my, int mz) {
   return false;
 }
 
-template <typename V, int MY, int MZ, int NY, int NZ>
+template <typename V, int MY, int MZ>
 static vie_status launch_pass_b_reg(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* twy,
                                     const V* twz, cudaStream_t s) {
   constexpr int PY = (MY % 2 == 0) ? MY + 1 : MY;
   constexpr int PZ = (MZ % 2 == 0) ? MZ + 1 : MZ;
   const size_t smem = (size_t)(MY + MZ + 3 * MZ * PY + 3 * g.ny * PZ + 6 * g.Kz * g.Ky) * sizeof(V);
   if (smem > 220 * 1024) { set_error("pass B shared memory %zu too large", smem); return VIE_ERR_INVALID; }
-  VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_reg_kernel<V, MY, MZ, NY, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_reg_kernel<V, MY, MZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)smem));
   int lines = 3 * (g.ny > MZ ? g.ny : MZ);
   int threads = ((lines + 31) / 32) * 32;
   if (threads > 256) threads = 256;
-  VIE_CUDA_TRY(launch_pdl(pass_b_reg_kernel<V, MY, MZ, NY, NZ>, dim3((unsigned)g.Mx, (unsigned)count), dim3(threads), smem,
+  VIE_CUDA_TRY(launch_pdl_if(b_starts_early<V>(g, count), pass_b_reg_kernel<V, MY, MZ>, dim3((unsigned)g.Mx, (unsigned)count), dim3(threads), smem,
                           s, pp, g, twy, twz));
   return VIE_OK;
 }
 
 // complex128 lines longer than 30 would spill registers: those keep the generic pass
-template <typename V, int MY, int MZ, int NY = 0, int NZ = 0>
+template <typename V, int MY, int MZ>
 static vie_status try_pass_b_reg(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* twy,
                                  const V* twz, cudaStream_t s, bool* done) {
   if constexpr (sizeof(V) == sizeof(float2) || (MY <= 30 && MZ <= 30)) {
     *done = true;
-    return launch_pass_b_reg<V, MY, MZ, NY, NZ>(pp, count, g, twy, twz, s);
+    return launch_pass_b_reg<V, MY, MZ>(pp, count, g, twy, twz, s);
   } else {
     *done = false;
     return VIE_OK;
@@ -674,11 +670,7 @@ static vie_status dispatch_pass_b_reg(const PassPtrs<V>& pp, int count, const Pa
   *done = false;
 #define VIE_X(a, b) \
   if (g.My == a && g.Mz == b) return try_pass_b_reg<V, a, b>(pp, count, g, twy, twz, s, done);
-#define VIE_Y(a, b, c, d)                       \
-  if (g.My == a && g.Mz == b && g.ny == c && g.nz == d) \
-    return try_pass_b_reg<V, a, b, c, d>(pp, count, g, twy, twz, s, done);
-  VIE_PASS_B_REG_FIXED(VIE_Y)
-#undef VIE_Y
+  if (b_any_compiled(g)) return VIE_OK;   // launch_b_any's kernel for this plane is the faster one
   VIE_PASS_B_REG_SIZES(VIE_X)
 #undef VIE_X
   return VIE_OK;
@@ -1389,164 +1381,6 @@ __global__ void __launch_bounds__(256) pass_b_jm_kernel(V* __restrict__ work, co
   }
 }
 
-// The JM-VIE pass B with register FFTs (as pass_b_reg_kernel, six
-// components): one CTA per kx, z and y lines of the six components in
-// registers, the N spectrum and the curl spectra of this kx staged in shared
-// memory while the forward transforms run.
-template <typename V, int MY, int MZ, int NY, int NZ>
-__global__ void __launch_bounds__(256) pass_b_reg_jm_kernel(V* __restrict__ work, const V* __restrict__ ghat,
-                                                            const V* __restrict__ chat, PassBGeom g,
-                                                            const V* __restrict__ twyg, const V* __restrict__ twzg,
-                                                            double kappa) {
-  typedef typename real_of<V>::type R;
-  constexpr int PY = (MY % 2 == 0) ? MY + 1 : MY;
-  constexpr int PZ = (MZ % 2 == 0) ? MZ + 1 : MZ;
-  extern __shared__ unsigned char smem_raw[];
-  V* twy = reinterpret_cast<V*>(smem_raw);
-  V* twz = twy + MY;
-  V* S1 = twz + MZ;
-  V* S2 = S1 + 6 * MZ * PY;
-  V* Gs = S2 + 6 * g.ny * PZ;          // N spectrum chunk (6 Kz Ky), then the curl chunk (3 Kz Ky)
-  const int kx = blockIdx.x;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int ny = NY > 0 ? NY : g.ny, nz = NZ > 0 ? NZ : g.nz;
-  const bool fx = kx > g.Mx - kx;
-  const int kxf = fx ? g.Mx - kx : kx;
-  const int cs = g.Kz * g.Ky;
-  pdl_launch_dependents();
-  for (int i = tid; i < MY; i += nth) __pipeline_memcpy_async(twy + i, twyg + i, sizeof(V));
-  for (int i = tid; i < MZ; i += nth) __pipeline_memcpy_async(twz + i, twzg + i, sizeof(V));
-  __pipeline_commit();
-  {
-    const V* G = ghat + (size_t)kxf * 6 * cs;
-    const V* C = chat + (size_t)kxf * 3 * cs;
-    for (int i = tid; i < 6 * cs; i += nth) __pipeline_memcpy_async(Gs + i, G + i, sizeof(V));
-    for (int i = tid; i < 3 * cs; i += nth) __pipeline_memcpy_async(Gs + 6 * cs + i, C + i, sizeof(V));
-    __pipeline_commit();
-  }
-  pdl_wait();
-  __pipeline_wait_prior(1);
-  __syncthreads();
-  V* slab = work + (size_t)kx * g.NL;
-  for (int line = tid; line < 6 * ny; line += nth) {
-    const int c = line / ny, y = line - c * ny;
-    V a[MZ];
-#pragma unroll
-    for (int z = 0; z < MZ; ++z) a[z] = (z < nz) ? slab[(c * nz + z) * ny + y] : zero_c<V>();
-    reg_fft<V, false, MZ>(a, twz);
-#pragma unroll
-    for (int kz = 0; kz < MZ; ++kz) S1[(c * MZ + kz) * PY + y] = a[kz];
-  }
-  __syncthreads();
-  for (int line = tid; line < 6 * MZ; line += nth) {
-    V a[MY];
-#pragma unroll
-    for (int y = 0; y < MY; ++y) a[y] = (y < ny) ? S1[line * PY + y] : zero_c<V>();
-    reg_fft<V, false, MY>(a, twy);
-#pragma unroll
-    for (int ky = 0; ky < MY; ++ky) S1[line * PY + ky] = a[ky];
-  }
-  __pipeline_wait_prior(0);
-  __syncthreads();
-  {
-    const V* G = Gs;
-    const V* Cc = Gs + 6 * cs;
-    const R kap = (R)kappa;
-    for (int e = tid; e < MZ * MY; e += nth) {
-      const int kz = e / MY, ky = e - kz * MY;
-      const bool fy = ky > MY - ky, fz = kz > MZ - kz;
-      const int kyf = fy ? MY - ky : ky, kzf = fz ? MZ - kz : kz;
-      const int o = kzf * g.Ky + kyf;
-      V gxx = G[o], gyy = G[cs + o], gzz = G[2 * cs + o];
-      V gxy = G[3 * cs + o], gxz = G[4 * cs + o], gyz = G[5 * cs + o];
-      if (fx ^ fy) gxy = scale(gxy, (R)-1);
-      if (fx ^ fz) gxz = scale(gxz, (R)-1);
-      if (fy ^ fz) gyz = scale(gyz, (R)-1);
-      V cx = Cc[o], cy = Cc[cs + o], cz = Cc[2 * cs + o];
-      if (fx) cx = scale(cx, (R)-1);
-      if (fy) cy = scale(cy, (R)-1);
-      if (fz) cz = scale(cz, (R)-1);
-      cx = scale(mul_pi(cx), kap);
-      cy = scale(mul_pi(cy), kap);
-      cz = scale(mul_pi(cz), kap);
-      V u[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) u[c] = S1[(c * MZ + kz) * PY + ky];
-      const V te0 = add(add(mul(gxx, u[0]), mul(gxy, u[1])), mul(gxz, u[2]));
-      const V te1 = add(add(mul(gxy, u[0]), mul(gyy, u[1])), mul(gyz, u[2]));
-      const V te2 = add(add(mul(gxz, u[0]), mul(gyz, u[1])), mul(gzz, u[2]));
-      const V tm0 = add(add(mul(gxx, u[3]), mul(gxy, u[4])), mul(gxz, u[5]));
-      const V tm1 = add(add(mul(gxy, u[3]), mul(gyy, u[4])), mul(gyz, u[5]));
-      const V tm2 = add(add(mul(gxz, u[3]), mul(gyz, u[4])), mul(gzz, u[5]));
-      S1[(0 * MZ + kz) * PY + ky] = sub(te0, sub(mul(cy, u[5]), mul(cz, u[4])));
-      S1[(1 * MZ + kz) * PY + ky] = sub(te1, sub(mul(cz, u[3]), mul(cx, u[5])));
-      S1[(2 * MZ + kz) * PY + ky] = sub(te2, sub(mul(cx, u[4]), mul(cy, u[3])));
-      S1[(3 * MZ + kz) * PY + ky] = add(tm0, sub(mul(cy, u[2]), mul(cz, u[1])));
-      S1[(4 * MZ + kz) * PY + ky] = add(tm1, sub(mul(cz, u[0]), mul(cx, u[2])));
-      S1[(5 * MZ + kz) * PY + ky] = add(tm2, sub(mul(cx, u[1]), mul(cy, u[0])));
-    }
-  }
-  __syncthreads();
-  for (int line = tid; line < 6 * MZ; line += nth) {
-    const int c = line / MZ, kz = line - c * MZ;
-    V a[MY];
-#pragma unroll
-    for (int ky = 0; ky < MY; ++ky) a[ky] = S1[line * PY + ky];
-    reg_fft<V, true, MY>(a, twy);
-#pragma unroll
-    for (int y = 0; y < MY; ++y)
-      if (y < ny) S2[(c * ny + y) * PZ + kz] = a[y];
-  }
-  __syncthreads();
-  for (int line = tid; line < 6 * ny; line += nth) {
-    const int c = line / ny, y = line - c * ny;
-    V a[MZ];
-#pragma unroll
-    for (int kz = 0; kz < MZ; ++kz) a[kz] = S2[line * PZ + kz];
-    reg_fft<V, true, MZ>(a, twz);
-#pragma unroll
-    for (int z = 0; z < MZ; ++z)
-      if (z < nz) slab[(c * nz + z) * ny + y] = a[z];
-  }
-}
-
-template <typename V, int MY, int MZ, int NY, int NZ>
-static vie_status try_pass_b_reg_jm(V* work, const V* ghat, const V* chat, const PassBGeom& g, const V* twy,
-                                    const V* twz, double kappa, cudaStream_t s, bool* done) {
-  *done = false;
-  // complex128 lines of these lengths would spill registers (the six-current
-  // multiply holds 12 spectra): those keep the generic JM pass
-  if constexpr (sizeof(V) == sizeof(float2)) {
-    constexpr int PY = (MY % 2 == 0) ? MY + 1 : MY;
-    constexpr int PZ = (MZ % 2 == 0) ? MZ + 1 : MZ;
-    const size_t smem = (size_t)(MY + MZ + 6 * MZ * PY + 6 * g.ny * PZ + 9 * g.Kz * g.Ky) * sizeof(V);
-    if (smem > 220 * 1024) return VIE_OK;
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_reg_jm_kernel<V, MY, MZ, NY, NZ>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int lines = 6 * (g.ny > MZ ? g.ny : MZ);
-    int threads = ((lines + 31) / 32) * 32;
-    if (threads > 256) threads = 256;
-    VIE_CUDA_TRY(launch_pdl(pass_b_reg_jm_kernel<V, MY, MZ, NY, NZ>, dim3((unsigned)g.Mx), dim3(threads), smem, s,
-                            work, ghat, chat, g, twy, twz, kappa));
-    *done = true;
-  }
-  return VIE_OK;
-}
-
-// register JM pass B for the compiled cross-sections (the guide's 23 x 11
-// with My 45 or 48 and Mz 24)
-template <typename V>
-static vie_status dispatch_pass_b_reg_jm(V* work, const V* ghat, const V* chat, const PassBGeom& g, const V* twy,
-                                         const V* twz, double kappa, cudaStream_t s, bool* done) {
-  *done = false;
-#define VIE_Y(a, b, c, d)                                  \
-  if (g.My == a && g.Mz == b && g.ny == c && g.nz == d)     \
-    return try_pass_b_reg_jm<V, a, b, c, d>(work, ghat, chat, g, twy, twz, kappa, s, done);
-  VIE_PASS_B_REG_FIXED(VIE_Y)
-#undef VIE_Y
-  return VIE_OK;
-}
-
 // One line of `len` values at a[0], a[stride], ...: gathered into the warp's
 // scratch pair (sa, sb), transformed with Stockham stages by the 32 lanes of
 // the warp (warp-synchronous), scattered back.  Every lane of the warp calls
@@ -1702,8 +1536,6 @@ static vie_status run_jm(vie_plan* p, const V* x, V* y, const V* ghat, const V* 
   vie_status st = launch_x<V>(true, 0, p->ax[0], pp, 1, nx, NL, NL, twx, mode, s, NL);
   if (st != VIE_OK) return st;
   PassBGeom g{ny, nz, NL, Mx, My, Mz, p->kf[1], p->kf[2]};
-  st = dispatch_pass_b_reg_jm<V>((V*)p->jm_work, ghat, chat, g, twy, twz, p->kappa, s, &done);
-  if (st != VIE_OK) return st;
   if (!done) {
     st = launch_b_any<V>(pp, 1, g, 6, chat, p->kappa, twy, s, &done);
     if (st != VIE_OK) return st;

@@ -37,6 +37,15 @@ struct PassBGeom {
   int ny, nz, NL, Mx, My, Mz, Ky, Kz;
 };
 
+// Whether pass B may start while the x pass before it still runs.  Blocks that
+// start early crowd onto the SMs the x pass leaves idle; complex128 planes are
+// bound by the SM's FP64 rate, so with no more than two planes an SM that
+// costs more than the overlap gives (73 x 11 x 9, 150 planes: 151 us an
+// application against 83).
+template <typename V> inline bool b_starts_early(const PassBGeom& g, int count) {
+  return sizeof(V) == sizeof(float2) || (long)g.Mx * count > 2 * kSMs;
+}
+
 // x pass (or the split pass B's y passes) for lines of n values and length
 // len, with register butterflies of run-time radices.  nyz: voxels of the
 // cross-section (the contrast row of a line is line % nyz); gsz: lines of a
@@ -45,6 +54,13 @@ struct PassBGeom {
 template <typename V>
 vie_status launch_x_any(bool forward, const PassPtrs<V>& pp, int count, int n, int nyz, int NL, int len, const V* tw,
                         int mode, cudaStream_t s, int gsz, bool* done);
+
+// Planes whose sizes are compiled into launch_b_any's complex64 kernel: the
+// 460 x 220 nm strip at 20 nm (23 x 11 voxels) in its smallest 5-smooth
+// embeddings.
+inline bool b_any_compiled(const PassBGeom& g) {
+  return g.ny == 23 && g.nz == 11 && g.Mz == 24 && (g.My == 45 || g.My == 48);
+}
 
 // Pass B on one CTA per kx with run-time radices: nc = 3 (J-VIE) or 6
 // (JM-VIE: pp.work[0], pp.ghat[0], chat and kappa, one problem).  *done =
