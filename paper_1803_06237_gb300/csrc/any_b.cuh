@@ -95,18 +95,6 @@ __device__ __forceinline__ void with_r2(int r, F&& f) {
   }
 }
 
-// a[z] times exp(-/+ 2 pi i z / L), z < L / 2 (the odd frequencies' input, or
-// the conjugate on their output)
-template <typename V, bool INV, int L>
-__device__ __forceinline__ void half_twiddle(V (&a)[L / 2]) {
-  typedef typename real_of<V>::type T;
-  static_for<1, L / 2>([&](auto zc) {
-    constexpr int z = decltype(zc)::value;
-    typedef TwConst<L, z> W;
-    a[z] = mul_cs(a[z], (T)W::c, INV ? -(T)W::s : (T)W::s);
-  });
-}
-
 template <typename V, int NC, bool STAGE, bool SMALL, typename FIX>
 __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && NC == 3 ? 3 : 2) : 1) pass_b_any_kernel(
     const __grid_constant__ PassPtrs<V> pp, const V* __restrict__ chat, double kappa, PassBGeom g, BAny q,

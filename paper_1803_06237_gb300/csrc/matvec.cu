@@ -343,18 +343,122 @@ static vie_status launch_pass_b_cluster(const PassPtrs<V>& pp, int count, const 
 // A B2 block takes one folded kxf, kBzCells consecutive folded kyf and all
 // their images (kx, Mx - kx) x (ky, My - ky): four contiguous runs of Y,
 // and each folded spectrum entry is read from memory once per block and
-// serves up to 8 spectral cells (kz and Mz - kz lie in the same thread's
-// line).  Threads (c, cell) transform one
-// component's z-line; the multiply exchanges them through shared memory.
+// serves up to 8 spectral cells (kz and Mz - kz lie in the same line).
 // ---------------------------------------------------------------------------
 constexpr int kBzCells = 16;
 constexpr int kBzThreads = 3 * 4 * kBzCells;
 
+// complex64: one thread takes a cell's three lines through forward transform,
+// product and inverse transform without leaving its registers; shared memory
+// only regroups the lines between global memory and the threads.  Half of a
+// line's inputs are padding and half of its outputs are cropped, so for even
+// MZ the radix-2 step falls apart into the even and the odd frequencies, MZ / 2
+// points each, taken one after the other (half the registers, 16 to 24
+// products each).  With a thread per component's line the lines went through
+// shared memory four times more, for the product and back: bound by that and
+// by its barriers, 455 us against 334 for 1600 x 1200 cells of 11 values into 24
+// (1.3 GB: 190 us at the copy rate).  Five or six blocks an SM by registers.
+// NZ > 0 fixes nz at compile time; NZ = 0 reads it from g.  mnl3: division by
+// 3 nz (any e < 2^16: e umulhi ceil(2^32 / 3 nz)).
+template <int MZ, int NZ>
+__global__ void __launch_bounds__(4 * kBzCells, MZ <= 12 || MZ == 16 || NZ == 11 ? 6 : MZ <= 24 ? 5 : 4)
+    pass_bz_cells_kernel(const __grid_constant__ PassPtrs<float2> pp, PassBGeom g, int tiles, unsigned mnl3) {
+  if (skip_problem(pp)) return;
+  typedef float2 V;
+  constexpr int C4 = 4 * kBzCells, KZ = MZ / 2 + 1;
+  const int nz = NZ > 0 ? NZ : g.nz, nl3 = 3 * nz, pio = nl3 | 1;
+  auto by_nl3 = [&](int e) { return NZ > 0 ? e / (3 * (NZ > 0 ? NZ : 1)) : (int)__umulhi((unsigned)e, mnl3); };
+  extern __shared__ unsigned char smem_raw[];
+  long long* base = reinterpret_cast<long long*>(smem_raw);   // Y offset of each cell, -1: no cell
+  V* Gs = reinterpret_cast<V*>(base + C4);                    // [comp][kzf][j]: 6 KZ kBzCells
+  V* IO = Gs + (size_t)6 * KZ * kBzCells;                     // [cell][pio]
+  const int kxf = blockIdx.x / tiles;
+  const int kyf0 = (blockIdx.x - kxf * tiles) * kBzCells;
+  const int tid = threadIdx.x;                                // the thread's cell: image * kBzCells + j
+  const int img = tid / kBzCells, j = tid - img * kBzCells;
+  pdl_launch_dependents();
+  // the spectrum tile is the plan's: loaded before the dependency wait
+  {
+    const V* G = pp.ghat[blockIdx.y] + (size_t)kxf * 6 * KZ * g.Ky;
+    if (kyf0 + j < g.Ky)
+      for (int row = img; row < 6 * KZ; row += 4)              // row = comp KZ + kzf
+        __pipeline_memcpy_async(Gs + row * kBzCells + j, G + (size_t)row * g.Ky + kyf0 + j, sizeof(V));
+  }
+  // image: (kx, ky) = (kxf or Mx - kxf, kyf or My - kyf); no cell where an
+  // image repeats another (kxf = 0 or Mx / 2, same for y) or kyf lies past the
+  // folded range
+  const int kyf = kyf0 + j;
+  const bool valid = kyf < g.Ky && !((img & 1) && (kxf == 0 || 2 * kxf == g.Mx)) &&
+                     !((img & 2) && (kyf == 0 || 2 * kyf == g.My));
+  const int kx = (img & 1) ? g.Mx - kxf : kxf, ky = (img & 2) ? g.My - kyf : kyf;
+  base[tid] = valid ? ((long long)kx * g.My + ky) * nl3 : -1;
+  __syncthreads();
+  pdl_wait();
+  V* __restrict__ Y = pp.work2[blockIdx.y];
+  for (int e = tid; e < C4 * nl3; e += C4) {   // all loads in flight at once
+    const int cell = by_nl3(e), l = e - cell * nl3;
+    const long long b = base[cell];
+    if (b >= 0) __pipeline_memcpy_async(IO + cell * pio + l, Y + b + l, sizeof(V));
+  }
+  __pipeline_commit();
+  __pipeline_wait_prior(0);
+  __syncthreads();
+  if (valid) {
+    constexpr int P = MZ % 2 == 0 ? 2 : 1, M = MZ / P, H = (MZ + 1) / 2;   // H: most inputs of a line
+    constexpr int NI = NZ > 0 ? NZ : H;
+    const float sx = kx > g.Mx - kx ? -1.f : 1.f, sy = ky > g.My - ky ? -1.f : 1.f;
+    V* io = IO + tid * pio;
+    V keep[3][P == 2 ? H : 1];
+    static_for<0, P>([&](auto hc) {
+      constexpr int h = decltype(hc)::value;
+      V a[3][M];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int z = 0; z < M; ++z) a[c][z] = (z < NI && z < nz) ? io[c * nz + z] : zero_c<V>();
+        if constexpr (h == 1) half_twiddle<V, false, 2 * M>(a[c]);
+        reg_fft<V, false, M, P == 2 ? M : H>(a[c], nullptr);
+      }
+      static_for<0, M>([&](auto kc) {
+        constexpr int k = decltype(kc)::value, kz = P * k + h;
+        constexpr bool fz = kz > MZ - kz;
+        constexpr int gcs = KZ * kBzCells;
+        const V* Gc = Gs + (fz ? MZ - kz : kz) * kBzCells + j;
+        const V gxx = Gc[0], gyy = Gc[gcs], gzz = Gc[2 * gcs];
+        const V gxy = scale(Gc[3 * gcs], sx * sy), gxz = scale(Gc[4 * gcs], fz ? -sx : sx),
+                gyz = scale(Gc[5 * gcs], fz ? -sy : sy);
+        const V wx = a[0][k], wy = a[1][k], wz = a[2][k];
+        a[0][k] = add(add(mul(gxx, wx), mul(gxy, wy)), mul(gxz, wz));
+        a[1][k] = add(add(mul(gxy, wx), mul(gyy, wy)), mul(gyz, wz));
+        a[2][k] = add(add(mul(gxz, wx), mul(gyz, wy)), mul(gzz, wz));
+      });
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        reg_fft<V, true, M>(a[c], nullptr);
+        if constexpr (h == 1) half_twiddle<V, true, 2 * M>(a[c]);
+#pragma unroll
+        for (int z = 0; z < NI; ++z) {
+          if constexpr (h < P - 1) keep[c][z] = a[c][z];
+          else if (z < nz) io[c * nz + z] = P == 2 ? add(keep[c][P == 2 ? z : 0], a[c][z]) : a[c][z];
+        }
+      }
+    });
+  }
+  __syncthreads();
+  for (int e = tid; e < C4 * nl3; e += C4) {
+    const int cell = by_nl3(e), l = e - cell * nl3;
+    const long long b = base[cell];
+    if (b >= 0) Y[b + l] = IO[cell * pio + l];
+  }
+}
+
+// complex128: a thread per component's line (three lines of a cell and their
+// product do not fit a thread's registers; bound by FP64).
 // NZ > 0 fixes nz at compile time (the zero padding is not loaded and the
 // cropped outputs are dead code; the additions of the padding zeros stay,
 // since IEEE arithmetic keeps x + 0); NZ = 0 reads it from g.
 template <typename V, int MZ, int NZ>
-__global__ void __launch_bounds__(kBzThreads, sizeof(V) == sizeof(float2) ? 4 : 1)
+__global__ void __launch_bounds__(kBzThreads)
     pass_bz_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g, int tiles, const V* __restrict__ twzg) {
   if (skip_problem(pp)) return;
   constexpr int C4 = 4 * kBzCells;
@@ -483,17 +587,24 @@ template <typename V, int MZ, int NZ>
 static vie_status launch_pass_bz(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* twz,
                                  cudaStream_t s) {
   constexpr int C4 = 4 * kBzCells;
-  const int pio = (3 * g.nz) | 1;
-  if (pio > 3 * MZ) { set_error("pass B2: nz = %d too large for Mz = %d", g.nz, MZ); return VIE_ERR_INVALID; }
-  const size_t smem = (size_t)C4 * (sizeof(long long) + sizeof(int)) +
-                      ((size_t)MZ + 6 * (size_t)(MZ / 2 + 1) * kBzCells + 3 * MZ * C4) * sizeof(V);
-  if (smem > 220 * 1024) { set_error("pass B2 shared memory %zu too large", smem); return VIE_ERR_INVALID; }
-  VIE_CUDA_TRY(cudaFuncSetAttribute(pass_bz_kernel<V, MZ, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  constexpr size_t spec = 6 * (size_t)(MZ / 2 + 1) * kBzCells;
+  const int nl3 = 3 * g.nz, pio = nl3 | 1;
+  if (g.nz > (MZ + 1) / 2) { set_error("pass B2: nz = %d too large for Mz = %d", g.nz, MZ); return VIE_ERR_INVALID; }
   const int tiles = (g.Ky + kBzCells - 1) / kBzCells;
-  const int Kx = g.Mx / 2 + 1;
-  VIE_CUDA_TRY(launch_pdl(pass_bz_kernel<V, MZ, NZ>, dim3((unsigned)(Kx * tiles), (unsigned)count), dim3(kBzThreads),
-                          smem, s, pp, g, tiles, twz));
+  const dim3 grid((unsigned)((g.Mx / 2 + 1) * tiles), (unsigned)count);
+  if constexpr (sizeof(V) == sizeof(float2)) {
+    const size_t smem = C4 * sizeof(long long) + (spec + (size_t)C4 * pio) * sizeof(V);
+    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_bz_cells_kernel<MZ, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
+    VIE_CUDA_TRY(launch_pdl(pass_bz_cells_kernel<MZ, NZ>, grid, dim3(C4), smem, s, pp, g, tiles,
+                            (unsigned)((0x100000000ull + nl3 - 1) / nl3)));
+  } else {
+    const size_t smem = (size_t)C4 * (sizeof(long long) + sizeof(int)) + (MZ + spec + 3 * MZ * C4) * sizeof(V);
+    if (smem > 220 * 1024) { set_error("pass B2 shared memory %zu too large", smem); return VIE_ERR_INVALID; }
+    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_bz_kernel<V, MZ, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem));
+    VIE_CUDA_TRY(launch_pdl(pass_bz_kernel<V, MZ, NZ>, grid, dim3(kBzThreads), smem, s, pp, g, tiles, twz));
+  }
   return VIE_OK;
 }
 

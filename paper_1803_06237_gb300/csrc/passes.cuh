@@ -39,11 +39,14 @@ struct PassBGeom {
 
 // Whether pass B may start while the x pass before it still runs.  Blocks that
 // start early crowd onto the SMs the x pass leaves idle; complex128 planes are
-// bound by the SM's FP64 rate, so with no more than two planes an SM that
-// costs more than the overlap gives (73 x 11 x 9, 150 planes: 151 us an
-// application against 83).
+// bound by the SM's FP64 rate, so where most of the grid is resident at once
+// that costs more than the overlap gives: up to two planes an SM (73 x 11 x 9,
+// 150 planes: 151 us an application against 83), and up to four small ones
+// (191 x 23 x 7, 384 planes of 45 x 15: 254 against 209; 180 x 27 x 9, 360 of
+// 54 x 18: 260 against 263).
 template <typename V> inline bool b_starts_early(const PassBGeom& g, int count) {
-  return sizeof(V) == sizeof(float2) || (long)g.Mx * count > 2 * kSMs;
+  const long planes = (long)g.Mx * count;
+  return sizeof(V) == sizeof(float2) || !(planes <= 2 * kSMs || (planes <= 4 * kSMs && g.My * g.Mz < 800));
 }
 
 // x pass (or the split pass B's y passes) for lines of n values and length

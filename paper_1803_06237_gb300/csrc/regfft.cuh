@@ -165,4 +165,16 @@ __device__ __forceinline__ void reg_fft(V (&a)[L], const V* __restrict__ tw) {
   RegStage<V, INV, L, L, 1, H>::run(a, tw);
 }
 
+// a[z] times exp(-/+ 2 pi i z / L), z < L / 2 (the odd frequencies' input, or
+// the conjugate on their output)
+template <typename V, bool INV, int L>
+__device__ __forceinline__ void half_twiddle(V (&a)[L / 2]) {
+  typedef typename real_of<V>::type T;
+  static_for<1, L / 2>([&](auto zc) {
+    constexpr int z = decltype(zc)::value;
+    typedef TwConst<L, z> W;
+    a[z] = mul_cs(a[z], (T)W::c, INV ? -(T)W::s : (T)W::s);
+  });
+}
+
 }  // namespace vie

@@ -62,3 +62,16 @@ def test_jm_operator(grid, dtype, tol):
     ref = jm.matvec(Gh, Ch, grid, op.contrast_M(op.chi_from_permittivity(eps, 2.085)), jm.mu_contrast(mu), u, kappa)
     got = y.cpu().numpy().astype(np.complex128)
     assert np.linalg.norm(got - ref.ravel()) <= tol * np.linalg.norm(ref)
+
+
+# planes too large for one CTA: every z length of the split pass B (5, 8, 9,
+# 12, 15, 15, 18, 20, 24, 24, 25, 27, 30, 32), with and without a middle kx, ky
+# that is its own image, last tiles of one to sixteen cells
+SPLIT = [(2, 961, 3), (3, 601, 4), (4, 545, 5), (2, 405, 6), (3, 325, 7), (4, 338, 8), (2, 270, 9), (3, 243, 10),
+         (4, 203, 11), (6, 211, 12), (2, 200, 13), (3, 182, 14), (4, 163, 15), (5, 152, 16)]
+
+
+@pytest.mark.parametrize("grid", SPLIT)
+@pytest.mark.parametrize("dtype,tol", [(np.complex64, 2e-6), (np.complex128, 1e-12)])
+def test_operator_on_large_planes(grid, dtype, tol):
+    test_operator_and_source(grid, dtype, tol)
