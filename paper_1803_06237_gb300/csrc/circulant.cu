@@ -15,11 +15,10 @@
 //      shared memory and transformed along k by a Stockham FFT (radices 2-5
 //      as butterflies, larger prime factors such as 7, 11, 13 summed
 //      directly), so the blocks c_k are never stored,
-//   3. LU with partial pivoting of the nx blocks W_hat(w): panels of nb
-//      columns factored in shared memory, row swaps, a triangular solve for
-//      the U row block, and the updates A22 -= L21 U12 as batched complex
-//      GEMMs in FP32: inside an outer block of 64 columns after every panel,
-//      on the trailing matrix once per outer block.
+//   3. LU with partial pivoting of the nx blocks W_hat(w): outer blocks of 64
+//      columns in left-looking panels of 16 held in registers, row swaps, one
+//      triangular solve for the block's rows and one update A22 -= L21 U12 of
+//      the trailing matrix per outer block, in FP32.
 // Application z = W^{-1} v (complex64):
 //   V_hat = FFT along x of the 3 ny nz lines, one pivoted forward and
 //   backward substitution per frequency (one CTA each, the factor streamed
@@ -39,7 +38,7 @@ struct vie_circulant {
   int device = 0;
   const vie_plan* plan = nullptr;
   int gen = 0;                 // contrast generation the factors were built from
-  int nx = 0, ny = 0, nz = 0, B = 0, R = 0, nb = 32;
+  int nx = 0, ny = 0, nz = 0, B = 0, R = 0;
   float2* W = nullptr;         // nx x R x R: LU factors (unit L below, U on and above the diagonal)
   __half2* W16 = nullptr;      // the same in complex half precision, as tiles (VIE_CIRC_FP16_FACTORS; W is then freed)
   bool fp16 = false;
@@ -222,72 +221,177 @@ __global__ void __launch_bounds__(256) lines_fft_kernel(const float2* __restrict
 // ---------------------------------------------------------------------------
 // batched LU with partial pivoting (row-major blocks, one matrix per CTA)
 // ---------------------------------------------------------------------------
-// Panel j0 .. j0 + nbe - 1 of every matrix, rows j0 .. R - 1, factored in
-// shared memory (pitch nbe + 1): per column the largest |a| below the
-// diagonal is the pivot (lowest row on ties), rows are swapped inside the
-// panel, the column is scaled by the pivot's inverse and the rest of the
-// panel gets the rank-1 update.  piv[j] = the row swapped with row j.
-__global__ void __launch_bounds__(256) lu_panel_kernel(float2* __restrict__ W, int R, int j0, int nbe,
-                                                       int* __restrict__ piv, int* __restrict__ flag) {
-  extern __shared__ float2 P[];
-  __shared__ float bval[8];
-  __shared__ int bidx[8];
-  __shared__ int ipiv;
+// An outer block of kOuter columns is factored in panels of kPanel, looking to
+// the left: a panel first takes up the products of the block's panels before
+// it, so that no column of the block is rewritten by them.
+constexpr int kOuter = 64;
+constexpr int kPanel = 16;
+constexpr int kMaxUnknowns = 1656;      // of a cross-section
+constexpr int kPanelRows = 7 * 256;     // a panel's rows in registers: up to 7 a thread
+static_assert(kMaxUnknowns <= kPanelRows, "the largest panel has no kernel");
+
+// acc - a b, four multiply-adds
+__device__ __forceinline__ void fnma(float2& acc, float2 a, float2 b) {
+  acc.x = fmaf(-a.x, b.x, fmaf(a.y, b.y, acc.x));
+  acc.y = fmaf(-a.x, b.y, fmaf(-a.y, b.x, acc.y));
+}
+
+// Panel j0 .. j0 + nbe - 1 of every matrix, rows j0 .. R - 1, one CTA a
+// matrix: the block's earlier panels J .. j0 - 1 are applied, then per column
+// the largest |a| below the diagonal is the pivot (lowest row on ties), rows
+// are swapped inside the panel, the column is scaled by the pivot's inverse
+// and the rest of the panel gets the rank-1 update.  piv[j] = the row swapped
+// with row j.  A thread keeps rows tid + 256 k of the panel in registers (RP
+// of them): a column costs two barriers, eight candidates and one broadcast
+// row.  Bound by those and by one CTA an SM; with the panel in shared memory
+// and its products with later columns as launches of their own, panels, those
+// products and triangular solves took 8.5 ms for 160 blocks of 1080 unknowns,
+// here 6.1 (396 blocks, the whole setup: 67 -> 58.5 ms).
+template <int RP>
+__global__ void __launch_bounds__(256, RP == 1 ? 3 : RP == 2 ? 2 : 1) lu_panel_kernel(
+    float2* __restrict__ W, int R, int J, int j0, int nbe, int* __restrict__ piv, int* __restrict__ flag) {
+  constexpr int NB = kPanel, NL = kOuter - kPanel;
+  __shared__ float2 Lb[NL][NL + 1];                // rows and columns J .. j0 - 1: unit lower triangle
+  __shared__ __align__(16) float2 U[NL][NB];       // rows J .. j0 - 1 of the panel's columns
+  __shared__ __align__(16) float2 prow[2][NB], srow[2][NB];
+  __shared__ float bval[2][8];
+  __shared__ int bidx[2][8];
   float2* A = W + (size_t)blockIdx.x * R * R;
-  const int rows = R - j0, pitch = nbe + 1;
-  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, wid = tid >> 5;
-  for (int e = tid; e < rows * nbe; e += nth) {
-    const int i = e / nbe, c = e - i * nbe;
-    P[i * pitch + c] = A[(size_t)(j0 + i) * R + j0 + c];
+  const int rows = R - j0, k0 = j0 - J;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  float2 a[RP][NB];
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    const int i = tid + 256 * k;
+    const float2* src = A + (size_t)(j0 + i) * R + j0;
+#pragma unroll
+    for (int c = 0; c < NB; ++c) a[k][c] = i < rows && c < nbe ? src[c] : make_float2(0.f, 0.f);
   }
-  __syncthreads();
-  for (int jj = 0; jj < nbe; ++jj) {
-    // pivot search over rows jj .. rows - 1 of column jj
-    float best = -1.f;
-    int bi = rows;
-    for (int i = jj + tid; i < rows; i += nth) {
-      const float2 a = P[i * pitch + jj];
-      const float m = a.x * a.x + a.y * a.y;
-      if (m > best) { best = m; bi = i; }
+  if (k0 > 0) {
+    for (int e = tid; e < k0 * k0; e += 256) {
+      const int i = e / k0, t = e - i * k0;
+      Lb[i][t] = A[(size_t)(J + i) * R + J + t];
     }
+    for (int e = tid; e < k0 * NB; e += 256) {
+      const int i = e / NB, c = e - i * NB;
+      U[i][c] = c < nbe ? A[(size_t)(J + i) * R + j0 + c] : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    // unit lower solve, two columns a warp, a lane per row of 16
+    const int c = 2 * wid + (lane >> 4), r = lane & 15;
+    for (int q = 0; q < k0; q += 16) {
+      float2 x = U[q + r][c];
+      for (int t = 0; t < q; ++t) fnma(x, Lb[q + r][t], U[t][c]);
+#pragma unroll
+      for (int t = 0; t < 15; ++t) {
+        const float2 xt = make_float2(__shfl_sync(0xffffffffu, x.x, t, 16), __shfl_sync(0xffffffffu, x.y, t, 16));
+        if (r > t) fnma(x, Lb[q + r][q + t], xt);
+      }
+      U[q + r][c] = x;
+      __syncwarp();
+    }
+    __syncthreads();
+    for (int e = tid; e < k0 * NB; e += 256) {
+      const int i = e / NB, c2 = e - i * NB;
+      if (c2 < nbe) A[(size_t)(J + i) * R + j0 + c2] = U[i][c2];
+    }
+    const float2* L[RP];
+#pragma unroll
+    for (int k = 0; k < RP; ++k) L[k] = A + (size_t)(j0 + min(tid + 256 * k, rows - 1)) * R + J;
+#pragma unroll 2
+    for (int t = 0; t < k0; ++t) {
+      float2 l[RP];
+#pragma unroll
+      for (int k = 0; k < RP; ++k) l[k] = L[k][t];
+#pragma unroll
+      for (int c2 = 0; c2 < NB; c2 += 2) {
+        const float4 u = *reinterpret_cast<const float4*>(&U[t][c2]);
+#pragma unroll
+        for (int k = 0; k < RP; ++k) {
+          fnma(a[k][c2], l[k], make_float2(u.x, u.y));
+          fnma(a[k][c2 + 1], l[k], make_float2(u.z, u.w));
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int jj = 0; jj < NB; ++jj) {
+    if (jj >= nbe) break;
+    const int s = jj & 1;
+    // pivot: rows jj .. rows - 1 of column jj, the lowest row on ties
+    float best = -1.f;
+    int ip = rows;
+#pragma unroll
+    for (int k = 0; k < RP; ++k) {
+      const int i = tid + 256 * k;
+      const float m = a[k][jj].x * a[k][jj].x + a[k][jj].y * a[k][jj].y;
+      if (i >= jj && i < rows && m > best) { best = m; ip = i; }
+    }
+#pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float ob = __shfl_down_sync(0xffffffffu, best, o);
-      const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      const int oi = __shfl_down_sync(0xffffffffu, ip, o);
+      if (ob > best || (ob == best && oi < ip)) { best = ob; ip = oi; }
     }
-    if (lane == 0) { bval[wid] = best; bidx[wid] = bi; }
+    if (lane == 0) { bval[s][wid] = best; bidx[s][wid] = ip; }
     __syncthreads();
-    if (tid == 0) {
-      float b = bval[0];
-      int ii = bidx[0];
-      for (int w = 1; w < (nth >> 5); ++w)
-        if (bval[w] > b || (bval[w] == b && bidx[w] < ii)) { b = bval[w]; ii = bidx[w]; }
-      if (!(b > 0.f)) { atomicExch(flag, 1); ii = jj; }
-      ipiv = ii;
-      piv[(size_t)blockIdx.x * R + j0 + jj] = j0 + ii;
+    best = bval[s][0];
+    ip = bidx[s][0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+      const float ob = bval[s][w];
+      const int oi = bidx[s][w];
+      if (ob > best || (ob == best && oi < ip)) { best = ob; ip = oi; }
     }
-    __syncthreads();
-    const int ip = ipiv;
-    if (ip != jj)
-      for (int c = tid; c < nbe; c += nth) {
-        const float2 t = P[jj * pitch + c];
-        P[jj * pitch + c] = P[ip * pitch + c];
-        P[ip * pitch + c] = t;
+    if (!(best > 0.f)) {
+      ip = jj;
+      if (tid == 0) atomicExch(flag, 1);
+    }
+    if (tid == 0) piv[(size_t)blockIdx.x * R + j0 + jj] = j0 + ip;
+#pragma unroll
+    for (int k = 0; k < RP; ++k)
+      if (tid + 256 * k == ip) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) prow[s][c] = a[k][c];
       }
+    if (tid == jj) {
+#pragma unroll
+      for (int c = 0; c < NB; ++c) srow[s][c] = a[0][c];
+    }
     __syncthreads();
-    const float2 d = P[jj * pitch + jj];
+    // the other buffers of s are written again two columns on, behind the next column's barriers
+    if (ip != jj) {
+#pragma unroll
+      for (int k = 0; k < RP; ++k)
+        if (tid + 256 * k == ip) {
+#pragma unroll
+          for (int c = 0; c < NB; ++c) a[k][c] = srow[s][c];
+        }
+      if (tid == jj) {
+#pragma unroll
+        for (int c = 0; c < NB; ++c) a[0][c] = prow[s][c];
+      }
+    }
+    const float2 d = prow[s][jj];
     const float dd = d.x * d.x + d.y * d.y;
     const float2 inv = dd > 0.f ? make_float2(d.x / dd, -d.y / dd) : make_float2(0.f, 0.f);
-    for (int i = jj + 1 + tid; i < rows; i += nth) {
-      const float2 l = cmul(P[i * pitch + jj], inv);
-      P[i * pitch + jj] = l;
-      for (int c = jj + 1; c < nbe; ++c) P[i * pitch + c] = csub_mul(P[i * pitch + c], l, P[jj * pitch + c]);
+#pragma unroll
+    for (int k = 0; k < RP; ++k) {
+      if (tid + 256 * k <= jj) continue;
+      const float2 l = cmul(a[k][jj], inv);
+      a[k][jj] = l;
+#pragma unroll
+      for (int c = jj + 1; c < NB; ++c) fnma(a[k][c], l, prow[s][c]);
     }
-    __syncthreads();
   }
-  for (int e = tid; e < rows * nbe; e += nth) {
-    const int i = e / nbe, c = e - i * nbe;
-    A[(size_t)(j0 + i) * R + j0 + c] = P[i * pitch + c];
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    const int i = tid + 256 * k;
+    if (i >= rows) continue;
+    float2* dst = A + (size_t)(j0 + i) * R + j0;
+#pragma unroll
+    for (int c = 0; c < NB; ++c)
+      if (c < nbe) dst[c] = a[k][c];
   }
 }
 
@@ -309,150 +413,115 @@ __global__ void __launch_bounds__(256) lu_swap_kernel(float2* __restrict__ W, in
   }
 }
 
-// U12 = L11^{-1} A12: rows j0 .. j0 + NB - 1, columns j0 + NB .. R - 1; L11
-// is the unit lower triangle of the factored panel.  One thread per column.
-template <int NB>
-__global__ void __launch_bounds__(256) lu_trsm_kernel(float2* __restrict__ W, int R, int j0) {
-  __shared__ float2 L[NB][NB + 1];
+// U12 = L11^{-1} A12 of an outer block: rows J .. J + kOuter - 1, the columns
+// right of the block; L11 is the block's unit lower triangle.  One thread per
+// column, 16 rows at a time in registers, the rows solved before in shared
+// memory.  (A launch per panel read and wrote the rows four times.)
+constexpr int kTrsmCols = 128;
+constexpr size_t kTrsmSmem = (kOuter * kOuter + (kOuter - 16) * kTrsmCols) * sizeof(float2);
+__global__ void __launch_bounds__(kTrsmCols) lu_trsm_kernel(float2* __restrict__ W, int R, int J) {
+  extern __shared__ __align__(16) float2 ts[];
+  float2* Lt = ts;                          // [t][i]
+  float2* xs = Lt + kOuter * kOuter;        // [t][column]
   float2* A = W + (size_t)blockIdx.x * R * R;
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int i = e / NB, t = e - i * NB;
-    L[i][t] = A[(size_t)(j0 + i) * R + j0 + t];
-  }
-  __syncthreads();
-  const int c = j0 + NB + blockIdx.y * blockDim.x + threadIdx.x;
-  if (c >= R) return;
-  float2 x[NB];
-#pragma unroll
-  for (int i = 0; i < NB; ++i) x[i] = A[(size_t)(j0 + i) * R + c];
-#pragma unroll
-  for (int i = 1; i < NB; ++i)
-#pragma unroll
-    for (int t = 0; t < i; ++t) x[i] = csub_mul(x[i], L[i][t], x[t]);
-#pragma unroll
-  for (int i = 0; i < NB; ++i) A[(size_t)(j0 + i) * R + c] = x[i];
-}
-
-// Update of a rectangle of every matrix (blockIdx.z): A[r0 .. r1)[c0 .. c1) -=
-// A[r0 .. r1)[j0 .. j0 + KB) A[j0 .. j0 + KB)[c0 .. c1), the products of one
-// panel's rank.  One CTA per 64 x 64 tile: the two operand panels are staged
-// in shared memory (the left one transposed), each of the 256 threads
-// accumulates 4 x 4 complex products (rows ty + 16 a, columns tx + 16 b, so
-// that a warp's stores cover 16 consecutive columns).  The regions read and
-// written are disjoint, so the update is in place.
-template <int KB>
-__global__ void __launch_bounds__(256) lu_update_kernel(float2* __restrict__ W, int R, int j0, int r0, int r1, int c0,
-                                                        int c1) {
-  __shared__ float2 As[KB][65];
-  __shared__ float2 Bs[KB][64];
-  float2* A = W + (size_t)blockIdx.z * R * R;
-  const int i0 = r0 + blockIdx.y * 64, k0 = c0 + blockIdx.x * 64;
   const int tid = threadIdx.x;
-  for (int e = tid; e < 64 * KB; e += 256) {
-    const int i = e / KB, k = e - i * KB;
-    As[k][i] = i0 + i < r1 ? A[(size_t)(i0 + i) * R + j0 + k] : make_float2(0.f, 0.f);
-  }
-  for (int e = tid; e < 64 * KB; e += 256) {
-    const int k = e >> 6, j = e & 63;
-    Bs[k][j] = k0 + j < c1 ? A[(size_t)(j0 + k) * R + k0 + j] : make_float2(0.f, 0.f);
+  for (int e = tid; e < kOuter * kOuter; e += kTrsmCols) {
+    const int i = e / kOuter, t = e - i * kOuter;
+    Lt[t * kOuter + i] = A[(size_t)(J + i) * R + J + t];
   }
   __syncthreads();
-  const int tx = tid & 15, ty = tid >> 4;
-  float2 acc[4][4];
+  const int c = J + kOuter + blockIdx.y * kTrsmCols + tid;
+  if (c >= R) return;
+#pragma unroll 1
+  for (int q = 0; q < kOuter; q += 16) {
+    float2 x[16];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int r = 0; r < 16; ++r) x[r] = A[(size_t)(J + q + r) * R + c];
+#pragma unroll 2
+    for (int t = 0; t < q; ++t) {
+      const float2 xt = xs[t * kTrsmCols + tid];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-#pragma unroll 4
-  for (int k = 0; k < KB; ++k) {
-    float2 av[4], bv[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) av[a] = As[k][ty + 16 * a];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) bv[b] = Bs[k][tx + 16 * b];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        acc[a][b].x = fmaf(av[a].x, bv[b].x, fmaf(-av[a].y, bv[b].y, acc[a][b].x));
-        acc[a][b].y = fmaf(av[a].x, bv[b].y, fmaf(av[a].y, bv[b].x, acc[a][b].y));
+      for (int r = 0; r < 16; r += 2) {
+        const float4 l = *reinterpret_cast<const float4*>(Lt + t * kOuter + q + r);
+        fnma(x[r], make_float2(l.x, l.y), xt);
+        fnma(x[r + 1], make_float2(l.z, l.w), xt);
       }
-  }
+    }
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int r = i0 + ty + 16 * a;
-    if (r >= r1) continue;
-    float2* row = A + (size_t)r * R;
+    for (int i = 1; i < 16; ++i)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int c = k0 + tx + 16 * b;
-      if (c < c1) {
-        float2 v = row[c];
-        v.x -= acc[a][b].x;
-        v.y -= acc[a][b].y;
-        row[c] = v;
-      }
+      for (int t = 0; t < i; ++t) fnma(x[i], Lt[(q + t) * kOuter + q + i], x[t]);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      A[(size_t)(J + q + r) * R + c] = x[r];
+      if (q + 16 < kOuter) xs[(q + r) * kTrsmCols + tid] = x[r];
     }
   }
 }
 
-// Trailing update of an outer block of kOuter columns, A22 -= L21 U12 with
-// L21 = A[j1 .. R)[j0 .. j1), U12 = A[j0 .. j1)[j1 .. R), j1 = j0 + kOuter.
-// FP32-bound: with the rank of one panel (16 or 32) every tile of A22 went
-// through memory once per 16 or 32 products, as long as the products took;
-// with 64 the products dominate.  128 x 64 tiles, 8 x 4 complex accumulators
-// a thread (12 shared loads for 128 multiply-adds), the next 16 of the 64
-// products' operands on their way into registers while 16 are summed.  160
-// blocks of 1080 unknowns: all updates 28.4 -> 19.2 ms, 15.1 ms (33 TFLOP/s)
-// of it here; three different register operands hold FP32 multiply-adds to
-// 50 TFLOP/s on this chip.
-constexpr int kOuter = 64;
+// Trailing update of an outer block, A22 -= L21 U12 with L21 = A[j1 .. R)[j0 ..
+// j1), U12 = A[j0 .. j1)[j1 .. R), j1 = j0 + kOuter.  FP32-bound: with the
+// rank of one panel every tile of A22 went through memory once per 16
+// products, as long as the products took; with 64 the products dominate.  128
+// x 64 tiles, 8 x 4 complex accumulators a thread, all 64 products' operands
+// on their way into shared memory at once (four groups, summed as they
+// arrive), the left ones transposed so that a thread's eight come in four
+// 16-byte loads.  160 blocks of 1080 unknowns: 13.8 ms, 36 TFLOP/s; 15.1 with
+// operands staged through registers 16 products ahead (three different
+// register operands hold FP32 multiply-adds to 50 TFLOP/s on this chip).
 constexpr int kUpdK = 16;
+constexpr int kUpdPitch = 130;
+constexpr size_t kTrailSmem = (size_t)kOuter * (kUpdPitch + 64) * sizeof(float2);
 __global__ void __launch_bounds__(256, 2) lu_trailing_kernel(float2* __restrict__ W, int R, int j0) {
-  __shared__ float2 As[2][kUpdK][129];
-  __shared__ float2 Bs[2][kUpdK][64];
+  extern __shared__ __align__(16) float2 us[];
+  float2* As = us;                          // [k][row]
+  float2* Bs = As + kOuter * kUpdPitch;     // [k][column]
   float2* A = W + (size_t)blockIdx.z * R * R;
   const int j1 = j0 + kOuter;
-  const int i0 = j1 + blockIdx.y * 128, k0 = j1 + blockIdx.x * 64;
+  const int i0 = j1 + blockIdx.y * 128, c0 = j1 + blockIdx.x * 64;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  // loads: left rows ty + 16 u, column tx of the chunk; right rows tid >> 6 + 4 u, column tid & 63
-  float2 ra[8], rb[4];
-  auto fetch = [&](int kc) {
+  // past the matrix's edge: zeros (bytes not copied are filled with zeros)
+#pragma unroll
+  for (int g = 0; g < kOuter; g += kUpdK) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int r = i0 + ty + 16 * u;
-      ra[u] = r < R ? A[(size_t)r * R + j0 + kc + tx] : make_float2(0.f, 0.f);
+      __pipeline_memcpy_async(As + (g + tx) * kUpdPitch + ty + 16 * u, A + (size_t)min(r, R - 1) * R + j0 + g + tx,
+                              sizeof(float2), r < R ? 0 : sizeof(float2));
     }
-    const int c = k0 + (tid & 63);
+    const int c = c0 + (tid & 63);
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      rb[u] = c < R ? A[(size_t)(j0 + kc + (tid >> 6) + 4 * u) * R + c] : make_float2(0.f, 0.f);
-  };
-  auto put = [&](int s) {
-#pragma unroll
-    for (int u = 0; u < 8; ++u) As[s][tx][ty + 16 * u] = ra[u];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) Bs[s][(tid >> 6) + 4 * u][tid & 63] = rb[u];
-  };
+    for (int u = 0; u < 4; ++u) {
+      const int k = g + (tid >> 6) + 4 * u;
+      __pipeline_memcpy_async(Bs + k * 64 + (tid & 63), A + (size_t)(j0 + k) * R + min(c, R - 1), sizeof(float2),
+                              c < R ? 0 : sizeof(float2));
+    }
+    __pipeline_commit();
+  }
+  // thread: rows 2 ty + 32 a + {0, 1}, columns tx + 16 b
   float2 acc[8][4];
 #pragma unroll
   for (int a = 0; a < 8; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-  fetch(0);
-  put(0);
-  __syncthreads();
 #pragma unroll 1
-  for (int kc = 0; kc < kOuter; kc += kUpdK) {
-    const int s = (kc / kUpdK) & 1;
-    if (kc + kUpdK < kOuter) fetch(kc + kUpdK);
+  for (int g = 0; g < kOuter; g += kUpdK) {
+    if (g == 0) __pipeline_wait_prior(3);
+    else if (g == kUpdK) __pipeline_wait_prior(2);
+    else if (g == 2 * kUpdK) __pipeline_wait_prior(1);
+    else __pipeline_wait_prior(0);
+    __syncthreads();
 #pragma unroll 4
-    for (int k = 0; k < kUpdK; ++k) {
+    for (int k = g; k < g + kUpdK; ++k) {
       float2 av[8], bv[4];
 #pragma unroll
-      for (int a = 0; a < 8; ++a) av[a] = As[s][k][ty + 16 * a];
+      for (int a = 0; a < 4; ++a) {
+        const float4 t = *reinterpret_cast<const float4*>(As + k * kUpdPitch + 2 * ty + 32 * a);
+        av[2 * a] = make_float2(t.x, t.y);
+        av[2 * a + 1] = make_float2(t.z, t.w);
+      }
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = Bs[s][k][tx + 16 * b];
+      for (int b = 0; b < 4; ++b) bv[b] = Bs[k * 64 + tx + 16 * b];
 #pragma unroll
       for (int a = 0; a < 8; ++a)
 #pragma unroll
@@ -461,17 +530,15 @@ __global__ void __launch_bounds__(256, 2) lu_trailing_kernel(float2* __restrict_
           acc[a][b].y = fmaf(av[a].x, bv[b].y, fmaf(av[a].y, bv[b].x, acc[a][b].y));
         }
     }
-    if (kc + kUpdK < kOuter) put(s ^ 1);
-    __syncthreads();
   }
 #pragma unroll
   for (int a = 0; a < 8; ++a) {
-    const int r = i0 + ty + 16 * a;
+    const int r = i0 + 2 * ty + 32 * (a >> 1) + (a & 1);
     if (r >= R) continue;
     float2* row = A + (size_t)r * R;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      const int c = k0 + tx + 16 * b;
+      const int c = c0 + tx + 16 * b;
       if (c < R) {
         float2 v = row[c];
         v.x -= acc[a][b].x;
@@ -868,38 +935,31 @@ static vie_status circ_build(vie_circulant* c, cudaStream_t s, size_t smem_max) 
   build_fft_kernel<<<(unsigned)((RR + tl - 1) / tl), 256, fft_smem, s>>>(p->toeplitz, Sp, Sm, nx, ny, nz, tl, c->rd,
                                                                         c->tw, c->W);
   CIRC_TRY(cudaGetLastError());
-  // LU of the nx blocks: panels of nb columns; within an outer block of kOuter
-  // columns a panel updates the rest of the block's columns and rows, the
-  // trailing matrix is updated once per outer block
-  const int nb = c->nb;
-  auto update = [&](int j0, int r0, int r1, int c0, int c1) {
-    if (r0 >= r1 || c0 >= c1) return;
-    const dim3 g((unsigned)((c1 - c0 + 63) / 64), (unsigned)((r1 - r0 + 63) / 64), (unsigned)nx);
-    if (nb == 32) lu_update_kernel<32><<<g, 256, 0, s>>>(c->W, R, j0, r0, r1, c0, c1);
-    else lu_update_kernel<16><<<g, 256, 0, s>>>(c->W, R, j0, r0, r1, c0, c1);
-  };
+  // LU of the nx blocks: within an outer block of kOuter columns the panels
+  // look to the left; the rows right of the block and the trailing matrix are
+  // updated once per outer block
+  CIRC_TRY(cudaFuncSetAttribute(lu_trsm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrsmSmem));
+  CIRC_TRY(cudaFuncSetAttribute(lu_trailing_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrailSmem));
   for (int J = 0; J < R; J += kOuter) {
     const int JE = min(J + kOuter, R);
-    for (int j0 = J; j0 < JE; j0 += nb) {
-      const int nbe = min(nb, R - j0), j1 = j0 + nbe;
-      const size_t smem = (size_t)(R - j0) * (nbe + 1) * sizeof(float2);
-      CIRC_TRY(cudaFuncSetAttribute(lu_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      lu_panel_kernel<<<nx, 256, smem, s>>>(c->W, R, j0, nbe, piv, c->flag);
-      lu_swap_kernel<<<dim3(nx, (R + 255) / 256), 256, 0, s>>>(c->W, R, j0, nbe, piv);
-      if (j1 < R) {
-        // here nbe == nb: only the last panel can be narrower, and nothing is right of it
-        const dim3 tg(nx, (R - j1 + 255) / 256);
-        if (nb == 32) lu_trsm_kernel<32><<<tg, 256, 0, s>>>(c->W, R, j0);
-        else lu_trsm_kernel<16><<<tg, 256, 0, s>>>(c->W, R, j0);
-        update(j0, j1, R, j1, JE);     // the block's remaining columns, every row
-        update(j0, j1, JE, JE, R);     // the block's remaining rows, the columns right of it
+    for (int j0 = J; j0 < JE; j0 += kPanel) {
+      const int nbe = min(kPanel, R - j0);
+      switch ((R - j0 + 255) / 256) {
+        case 1: lu_panel_kernel<1><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
+        case 2: lu_panel_kernel<2><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
+        case 3: lu_panel_kernel<3><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
+        case 4: lu_panel_kernel<4><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
+        case 5: lu_panel_kernel<5><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
+        default: lu_panel_kernel<kPanelRows / 256><<<nx, 256, 0, s>>>(c->W, R, J, j0, nbe, piv, c->flag); break;
       }
-      CIRC_TRY(cudaGetLastError());
+      lu_swap_kernel<<<dim3(nx, (R + 255) / 256), 256, 0, s>>>(c->W, R, j0, nbe, piv);
     }
+    CIRC_TRY(cudaGetLastError());
     if (JE < R) {
       const int n = R - JE;
-      lu_trailing_kernel<<<dim3((unsigned)((n + 63) / 64), (unsigned)((n + 127) / 128), (unsigned)nx), 256, 0, s>>>(
-          c->W, R, J);
+      lu_trsm_kernel<<<dim3((unsigned)nx, (unsigned)((n + kTrsmCols - 1) / kTrsmCols)), kTrsmCols, kTrsmSmem, s>>>(c->W, R, J);
+      lu_trailing_kernel<<<dim3((unsigned)((n + 63) / 64), (unsigned)((n + 127) / 128), (unsigned)nx), 256, kTrailSmem,
+                           s>>>(c->W, R, J);
       CIRC_TRY(cudaGetLastError());
     }
   }
@@ -948,6 +1008,9 @@ vie_status circulant_apply(vie_circulant* c, int dtype, const void* v, void* z, 
     VIE_CUDA_TRY(cudaFuncSetAttribute(circ_solve_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     circ_solve_tiles_kernel<<<nx, 256, smem, s>>>(c->W16, c->perm, c->vh, R, nb);
   } else {
+    // the vector and 37 KB of tiles: past 48 KB from 1408 unknowns on
+    VIE_CUDA_TRY(cudaFuncSetAttribute(circ_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(R * sizeof(float2))));
     circ_solve_kernel<<<nx, 256, (size_t)R * sizeof(float2), s>>>(c->W, c->perm, c->vh, R);
   }
   VIE_LAUNCH_CHECK();
@@ -982,10 +1045,7 @@ vie_status vie_circulant_create(vie_plan* plan, int flags, vie_circulant** out, 
   c->nz = plan->n[2];
   c->B = c->ny * c->nz;
   c->R = 3 * c->B;
-  // the panel (R rows x nb columns) must fit in shared memory
-  const size_t budget = 220 * 1024;
-  c->nb = (size_t)c->R * 33 * sizeof(float2) <= budget ? 32 : 16;
-  if ((size_t)c->R * 17 * sizeof(float2) > budget) {
+  if (c->R > kMaxUnknowns) {
     set_error("cross-section of %d unknowns is too large for the block-circulant preconditioner", c->R);
     delete c;
     return VIE_ERR_INVALID;

@@ -68,6 +68,15 @@ def test_apply_matches_oracle(grid, dtype, fp16):
     assert np.linalg.norm(z - z_ref) / np.linalg.norm(z_ref) < tol
 
 
+# edges of the factorisation: fewer unknowns than a panel, whole panels and
+# outer blocks of 64 and one or a few past them, one to seven rows a thread
+# (the last grid has the most unknowns that are taken: 1656)
+@pytest.mark.parametrize("grid", [(3, 1, 1), (4, 4, 4), (5, 7, 3), (4, 11, 2), (3, 8, 8), (3, 13, 5), (2, 12, 14),
+                                  (2, 19, 9), (3, 20, 18), (2, 21, 21), (2, 23, 24)])
+def test_factorisation_edges(grid):
+    test_apply_matches_oracle(grid, np.complex64, False)
+
+
 def test_zero_contrast_is_identity():
     grid = (12, 3, 2)
     plan = vie.vie_plan_create(grid, H, K0, EPS_BG)
