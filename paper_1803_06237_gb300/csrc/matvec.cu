@@ -738,13 +738,6 @@ __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__
 #define VIE_PASS_B_REG_SIZES(X) \
   X(24, 24) X(45, 24) X(48, 24) X(50, 24) X(30, 24) X(40, 24) X(25, 24) X(45, 25) X(48, 25) X(24, 25)
 
-bool pass_b_reg_available(int my, int mz) {
-#define VIE_X(a, b) if (my == a && mz == b) return true;
-  VIE_PASS_B_REG_SIZES(VIE_X)
-#undef VIE_X
-  return false;
-}
-
 template <typename V, int MY, int MZ>
 static vie_status launch_pass_b_reg(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* twy,
                                     const V* twz, cudaStream_t s) {
@@ -844,15 +837,15 @@ __global__ void __launch_bounds__(256) pass_c_kernel(const __grid_constant__ Pas
 // ---------------------------------------------------------------------------
 __host__ __device__ constexpr int pitch_mod16(int n, int lpb) { return n + ((lpb - n % 16) % 16 + 16) % 16; }
 
-// NX > 0 (a multiple of L1 for pass A, of L2 for pass C) fixes the line
-// length at compile time: the zero padding of the forward transform is not
-// loaded and the cropped outputs of the inverse are dead code (the additions
-// of the padding zeros stay: IEEE arithmetic keeps x + 0).
+// NX (a multiple of L1 and L2) is the line length, compiled in: the zero
+// padding of the forward transform is not loaded and the cropped outputs of the
+// inverse are dead code (the additions of the padding zeros stay: IEEE
+// arithmetic keeps x + 0).
 template <typename V, int L1, int L2, int LPB, int NX>
 __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_a4_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int NL, const V* __restrict__ twxg, int gsz) {
   if (skip_problem(pp)) return;
-  static_assert(NX == 0 || (NX % L1 == 0 && NX % L2 == 0), "compiled line length must divide by L1 and L2");
+  static_assert(NX % L1 == 0 && NX % L2 == 0, "compiled line length must divide by L1 and L2");
   const V* __restrict__ x = pp.x[blockIdx.y];
   V* __restrict__ work = pp.work[blockIdx.y];
   constexpr int MX = L1 * L2;
@@ -889,7 +882,7 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_a4_kernel(
 #pragma unroll
     for (int n2 = 0; n2 < L2; ++n2) {
       const int n = n1 + L1 * n2;
-      const bool in = NX > 0 ? (n2 < NX / L1) : (n < nx);
+      const bool in = n2 < NX / L1;
       a[n2] = (l < nl && in) ? Xs[l * P + n] : zero_c<V>();
     }
     reg_fft<V, false, L2>(a, tw2);
@@ -941,17 +934,13 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
     // FFTs; the contrast rows are plan data, x only after the dependency wait
     for (int i = tid; i < MX; i += nth) __pipeline_memcpy_async(twx + i, twxg + i, sizeof(V));
     __pipeline_commit();
-    if (mode != MODE_PLAIN) {
-      for (int l = 0; l < nl; ++l) {
-        const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
-        for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
-      }
+    for (int l = 0; l < nl; ++l) {
+      const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
+      for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
     }
     pdl_wait();
-    if (mode != MODE_PLAIN) {
-      const V* xsrc = x + (size_t)l0 * nx;
-      for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
-    }
+    const V* xsrc = x + (size_t)l0 * nx;
+    for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
     __pipeline_commit();
     __pipeline_wait_prior(1);      // twiddles only
   }
@@ -982,7 +971,7 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
 #pragma unroll
     for (int b1 = 0; b1 < L1; ++b1) {
       const int n = b2 + L2 * b1;
-      if (NX > 0 ? (b1 < NX / L2) : (n < nx)) Ys[l * P + n] = a[b1];
+      if (b1 < NX / L2) Ys[l * P + n] = a[b1];
     }
   }
   __syncthreads();
@@ -995,7 +984,6 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
     for (int e = tid; e < total; e += nth) {
       const int l = e / nx, ix = e - l * nx;
       const V uu = Ys[l * P + ix];
-      if (mode == MODE_PLAIN) { y[g0 + e] = uu; continue; }
       const V wv = Xs[e], mv = Ms[e];
       y[g0 + e] = (mode == MODE_OPERATOR) ? sub(wv, mul(mv, uu)) : mul(mv, sub(uu, wv));
     }
@@ -1013,8 +1001,8 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
 //   step 2: thread (l, n1, k3) transforms the L2 values over m2 and multiplies
 //           by w_Mx^(n1 kM);
 //   step 3: thread (l, kM) transforms the L1 values over n1.
-// LPB lines per block, lanes fastest over the lines.  NX > 0 fixes the line
-// length: the forward pass drops m3 >= NX / (L1 L2) (zero padding) and the
+// LPB lines per block, lanes fastest over the lines.  NX is the line length,
+// compiled in: the forward pass drops m3 >= NX / (L1 L2) (zero padding) and the
 // inverse pass keeps k1 < NX / M (the crop).  The inverse pass runs the same
 // steps with conjugate twiddles on spectrum index n (the workspace) and
 // spatial index k, then applies the contrast epilogue.
@@ -1067,7 +1055,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_a3_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int NL, const V* __restrict__ twxg, int gsz) {
   if (skip_problem(pp)) return;
   typedef X3<L1, L2, L3> G;
-  static_assert(NX == 0 || NX % (L1 * L2) == 0, "compiled line length must divide by L1 L2");
+  static_assert(NX % (L1 * L2) == 0, "compiled line length must divide by L1 L2");
   const V* __restrict__ x = pp.x[blockIdx.y];
   V* __restrict__ work = pp.work[blockIdx.y];
   constexpr int R1 = pitch_mod16(G::T1 * LPB, LPB);
@@ -1106,7 +1094,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_a3_kernel(
 #pragma unroll
     for (int m3 = 0; m3 < L3; ++m3) {
       const int n = n1 + L1 * (m2 + L2 * m3);
-      const bool in = NX > 0 ? (m3 < NX / (L1 * L2)) : (n < nx);
+      const bool in = m3 < NX / (L1 * L2);
       a[m3] = (l < nl && in) ? Xs[l * P + n] : zero_c<V>();
     }
   }
@@ -1133,7 +1121,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
     int gsz) {
   if (skip_problem(pp)) return;
   typedef X3<L1, L2, L3> G;
-  static_assert(NX == 0 || NX % G::M == 0, "compiled line length must divide by L2 L3");
+  static_assert(NX % G::M == 0, "compiled line length must divide by L2 L3");
   const V* __restrict__ work = pp.work[blockIdx.y];
   const V* __restrict__ x = pp.x[blockIdx.y];
   const V* __restrict__ Mc = pp.M[blockIdx.y];
@@ -1158,17 +1146,13 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
   {
     for (int i = tid; i < G::MX; i += nth) __pipeline_memcpy_async(twx + i, twxg + i, sizeof(V));
     __pipeline_commit();
-    if (mode != MODE_PLAIN) {
-      for (int l = 0; l < nl; ++l) {
-        const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
-        for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
-      }
+    for (int l = 0; l < nl; ++l) {
+      const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
+      for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
     }
     pdl_wait();
-    if (mode != MODE_PLAIN) {
-      const V* xsrc = x + (size_t)l0 * nx;
-      for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
-    }
+    const V* xsrc = x + (size_t)l0 * nx;
+    for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
     __pipeline_commit();
     __pipeline_wait_prior(1);      // twiddles only
   }
@@ -1197,7 +1181,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
 #pragma unroll
     for (int k1 = 0; k1 < L1; ++k1) {
       const int xo = kM + G::M * k1;
-      if (NX > 0 ? (k1 < NX / G::M) : (xo < nx)) Ys[l * P + xo] = c[k1];
+      if (k1 < NX / G::M) Ys[l * P + xo] = c[k1];
     }
   }
   __syncthreads();
@@ -1209,7 +1193,6 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
     for (int e = tid; e < total; e += nth) {
       const int l = e / nx, ix = e - l * nx;
       const V uu = Ys[l * P + ix];
-      if (mode == MODE_PLAIN) { y[g0 + e] = uu; continue; }
       const V wv = Xs[e], mv = Ms[e];
       y[g0 + e] = (mode == MODE_OPERATOR) ? sub(wv, mul(mv, uu)) : mul(mv, sub(uu, wv));
     }

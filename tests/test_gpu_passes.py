@@ -75,3 +75,10 @@ SPLIT = [(2, 961, 3), (3, 601, 4), (4, 545, 5), (2, 405, 6), (3, 325, 7), (4, 33
 @pytest.mark.parametrize("dtype,tol", [(np.complex64, 2e-6), (np.complex128, 1e-12)])
 def test_operator_on_large_planes(grid, dtype, tol):
     test_operator_and_source(grid, dtype, tol)
+
+
+# the cross-section with compiled strides (23 x 11 in 45 x 24), both operators
+def test_compiled_cross_section():
+    for dtype, tol in ((np.complex64, 2e-6), (np.complex128, 1e-12)):
+        test_operator_and_source((13, 23, 11), dtype, tol)
+        test_jm_operator((13, 23, 11), dtype, tol)
