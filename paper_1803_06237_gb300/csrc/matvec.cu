@@ -1338,7 +1338,15 @@ static vie_status run_passes(const vie_plan* p, const PassPtrs<V>& pp, int count
     st = launch_b_any<V>(pp, count, g, 3, nullptr, 0.0, twy, s, &done);
     if (st != VIE_OK) return st;
   }
-  if (!done && smem_b > 220 * 1024 && pp.work2[0] && pass_bz_available(Mz)) {
+  // complex64 planes that fit one block but have no split into the kernel's
+  // radices (My > 160, and a few others) take the split pass too where its
+  // buffer is there: the generic kernel's radices up to 5 make a dozen trips
+  // through shared memory on one block an SM (500 x 150 x 6: 507 us an
+  // application against 172; 800 x 170 x 6: 1129 against 223; 160 x 95 x 12:
+  // 289 against 87)
+  bool split = pass_bz_available(Mz) && (smem_b > 220 * 1024 || sizeof(V) == sizeof(float2));
+  for (int k = 0; k < count; ++k) split = split && pp.work2[k];
+  if (!done && split) {
     st = run_split_b<V>(p, pp, count, g, twy, twz, s);
     if (st != VIE_OK) return st;
     done = true;

@@ -71,7 +71,11 @@ SPLIT = [(2, 961, 3), (3, 601, 4), (4, 545, 5), (2, 405, 6), (3, 325, 7), (4, 33
          (4, 203, 11), (6, 211, 12), (2, 200, 13), (3, 182, 14), (4, 163, 15), (5, 152, 16)]
 
 
-@pytest.mark.parametrize("grid", SPLIT)
+# planes that fit one block in complex64 but have no split into its radices
+SPLIT_SMALL = [(5, 150, 6), (4, 95, 12), (3, 170, 7), (6, 81, 15), (2, 101, 11)]
+
+
+@pytest.mark.parametrize("grid", SPLIT + SPLIT_SMALL)
 @pytest.mark.parametrize("dtype,tol", [(np.complex64, 2e-6), (np.complex128, 1e-12)])
 def test_operator_on_large_planes(grid, dtype, tol):
     test_operator_and_source(grid, dtype, tol)
