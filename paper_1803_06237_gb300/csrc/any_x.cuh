@@ -252,7 +252,12 @@ static bool x_any_split(int len, bool small, XAny* g) {
       bool known = false;
       for (int r : kRadices) known |= r == r2;
       if (!known) continue;
-      const long cost = (r1 > 16 ? 1000000L : 0) + (r2 > 1 && !small ? 10000L : 0) + r1 * 100L + r1 + r2 + r3;
+      // a last radix of 4, without multiplications, beside larger even ones
+      // counts as 2 (200 x 200 x 11, 400 = 10 10 4: 103 us an application, 10
+      // 8 5: 115); beside odd ones it does not pay (162 x 162 x 11, 324 = 9 9 4:
+      // 97, 9 6 6: 75)
+      const int sum = r1 + r2 + (r3 == 4 && r2 > 1 && r1 % 2 == 0 && r2 % 2 == 0 ? 2 : r3);
+      const long cost = (r1 > 16 ? 1000000L : 0) + (r2 > 1 && !small ? 10000L : 0) + r1 * 100L + sum;
       if (best >= 0 && cost >= best) continue;
       best = cost;
       *g = XAny{len, r1, r2, r3, r2 * r3, r3 | 1, 0, 0, 0, div_magic(r2), div_magic(r3), 0};

@@ -71,8 +71,10 @@ SPLIT = [(2, 961, 3), (3, 601, 4), (4, 545, 5), (2, 405, 6), (3, 325, 7), (4, 33
          (4, 203, 11), (6, 211, 12), (2, 200, 13), (3, 182, 14), (4, 163, 15), (5, 152, 16)]
 
 
-# planes that fit one block in complex64 but have no split into its radices
-SPLIT_SMALL = [(5, 150, 6), (4, 95, 12), (3, 170, 7), (6, 81, 15), (2, 101, 11)]
+# planes that fit one block in complex64 but have no split into its radices; x
+# and y lines of 324 = 9 6 6 and 400 = 10 10 4
+SPLIT_SMALL = [(5, 150, 6), (4, 95, 12), (3, 170, 7), (6, 81, 15), (2, 101, 11), (162, 4, 3), (200, 162, 8),
+               (3, 200, 7)]
 
 
 @pytest.mark.parametrize("grid", SPLIT + SPLIT_SMALL)
