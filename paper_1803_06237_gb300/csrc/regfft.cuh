@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "fft.cuh"
+#include "twiddle.cuh"
 
 namespace vie {
 
@@ -22,26 +23,9 @@ __host__ __device__ constexpr bool reg_fft_supported(int n) {
   return n == 1 ? true : (first_radix(n) == 0 ? false : reg_fft_supported(n / first_radix(n)));
 }
 
-// exp(-2 pi i k / L) at compile time: the angle reduced to [-pi, pi], then
-// the Taylor series of cos and sin (30 terms: below 1e-16 for |x| <= pi).
-// The stages multiply by these constants, so no twiddle is loaded and
-// multiplications by 1, -i or (1 - i)/sqrt 2 fold.
-__host__ __device__ constexpr double tw_taylor(double x, bool want_sin) {
-  double term = want_sin ? x : 1.0, sum = term;
-  for (int n = want_sin ? 1 : 0; n < 60; n += 2) {
-    term *= -x * x / ((double)(n + 1) * (double)(n + 2));
-    sum += term;
-  }
-  return sum;
-}
-template <int L, int K>
-struct TwConst {
-  static constexpr int k = ((K % L) + L) % L;
-  static constexpr int kr = 2 * k > L ? k - L : k;    // angle in [-pi, pi]
-  static constexpr double x = -6.283185307179586476925286766559 * (double)kr / (double)L;
-  static constexpr double c = tw_taylor(x, false);
-  static constexpr double s = tw_taylor(x, true);
-};
+// The stages multiply by the compile-time constants TwConst, so no twiddle is
+// loaded and multiplications by 1 fold.
+
 // compile-time loop: f(std::integral_constant<int, I>) for I in [B, E)
 template <int B, int E, typename F>
 __device__ __forceinline__ void static_for(F&& f) {
