@@ -99,7 +99,6 @@ template <typename V, int NC, bool STAGE, bool SMALL, typename FIX>
 __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && NC == 3 ? 3 : 2) : 1) pass_b_any_kernel(
     const __grid_constant__ PassPtrs<V> pp, const V* __restrict__ chat, double kappa, PassBGeom g, BAny q,
     const V* __restrict__ twy) {
-  if (skip_problem(pp)) return;
   typedef typename real_of<V>::type R;
   constexpr int ZTOP = SMALL ? 24 : 32, R1TOP = SMALL ? 10 : 16, R2TOP = SMALL ? 6 : fused_max<V, NC>();
   extern __shared__ unsigned char smem_raw[];
@@ -127,7 +126,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
     G = Gs;
     Cc = Gs + 6 * cs;
   }
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   V* slab = pp.work[blockIdx.y] + (size_t)kx * g.NL;
   with_z<ZTOP, FIX>(Mz, [&](auto zc) {
     constexpr int MZ = decltype(zc)::value;

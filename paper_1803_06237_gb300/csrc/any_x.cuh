@@ -71,11 +71,8 @@ template <typename V, int TOP> __host__ __device__ constexpr int x_any_threads()
 template <typename V, int TOP>
 __global__ void __launch_bounds__(x_any_threads<V, TOP>(), 1) pass_a_any_kernel(const __grid_constant__ PassPtrs<V> pp, XAny g, int nx,
                                                          int NL, const V* __restrict__ tw, int gsz) {
-  // nothing to do before the wait: the flag is read behind it, as its writer
-  // may be the kernel before this one
   pdl_launch_dependents();
-  pdl_wait();
-  if (skip_problem(pp)) return;
+  if (skip_after_wait(pp)) return;
   extern __shared__ unsigned char smem_raw[];
   V* S = reinterpret_cast<V*>(smem_raw);
   const int lpb = g.lpb, t0 = div_by(threadIdx.x, g.ml), l = threadIdx.x - t0 * lpb, step = div_by(blockDim.x, g.ml);
@@ -147,11 +144,8 @@ template <typename V, int TOP>
 __global__ void __launch_bounds__(x_any_threads<V, TOP>(), 1) pass_c_any_kernel(const __grid_constant__ PassPtrs<V> pp, XAny g, int nx,
                                                          int nyz, int NL, const V* __restrict__ tw, int mode,
                                                          int gsz) {
-  // nothing to do before the wait: the flag is read behind it, as its writer
-  // may be the kernel before this one
   pdl_launch_dependents();
-  pdl_wait();
-  if (skip_problem(pp)) return;
+  if (skip_after_wait(pp)) return;
   extern __shared__ unsigned char smem_raw[];
   V* S = reinterpret_cast<V*>(smem_raw);
   const int lpb = g.lpb, t0 = div_by(threadIdx.x, g.ml), l = threadIdx.x - t0 * lpb, step = div_by(blockDim.x, g.ml);

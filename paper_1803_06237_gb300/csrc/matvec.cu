@@ -39,8 +39,7 @@ template <typename V>
 __global__ void __launch_bounds__(256) pass_a_kernel(const __grid_constant__ PassPtrs<V> pp, int nx, int NL,
                                                      Radices rx, const V* __restrict__ twg, int lines_per_block,
                                                      int gsz) {
-  if (skip_problem(pp)) return;
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   const V* __restrict__ x = pp.x[blockIdx.y];
   V* __restrict__ work = pp.work[blockIdx.y];
   extern __shared__ unsigned char smem_raw[];
@@ -73,8 +72,7 @@ template <typename V>
 __global__ void __launch_bounds__(256) pass_b_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g,
                                                      Radices ry, Radices rz, const V* __restrict__ twyg,
                                                      const V* __restrict__ twzg) {
-  if (skip_problem(pp)) return;
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   V* __restrict__ work = pp.work[blockIdx.y];
   const V* __restrict__ ghat = pp.ghat[blockIdx.y];
   extern __shared__ unsigned char smem_raw[];
@@ -182,7 +180,6 @@ __global__ void __launch_bounds__(256) pass_b_cluster_kernel(const __grid_consta
                                                              ClusterGeom q, Radices ry, Radices rz,
                                                              const V* __restrict__ twyg,
                                                              const V* __restrict__ twzg) {
-  if (skip_problem(pp)) return;
   namespace cgr = cooperative_groups;
   cgr::cluster_group cluster = cgr::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -203,7 +200,7 @@ __global__ void __launch_bounds__(256) pass_b_cluster_kernel(const __grid_consta
   pdl_launch_dependents();
   for (int i = tid; i < My; i += nth) twy[i] = twyg[i];
   for (int i = tid; i < Mz; i += nth) twz[i] = twzg[i];
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   V* __restrict__ slab = pp.work[blockIdx.y] + (size_t)kx * g.NL;
   const V* __restrict__ ghat = pp.ghat[blockIdx.y];
   for (int e = tid; e < nown * My; e += nth) {
@@ -364,7 +361,6 @@ constexpr int kBzThreads = 3 * 4 * kBzCells;
 template <int MZ, int NZ>
 __global__ void __launch_bounds__(4 * kBzCells, MZ <= 12 || MZ == 16 || NZ == 11 ? 6 : MZ <= 24 ? 5 : 4)
     pass_bz_cells_kernel(const __grid_constant__ PassPtrs<float2> pp, PassBGeom g, int tiles, unsigned mnl3) {
-  if (skip_problem(pp)) return;
   typedef float2 V;
   constexpr int C4 = 4 * kBzCells, KZ = MZ / 2 + 1;
   const int nz = NZ > 0 ? NZ : g.nz, nl3 = 3 * nz, pio = nl3 | 1;
@@ -394,7 +390,7 @@ __global__ void __launch_bounds__(4 * kBzCells, MZ <= 12 || MZ == 16 || NZ == 11
   const int kx = (img & 1) ? g.Mx - kxf : kxf, ky = (img & 2) ? g.My - kyf : kyf;
   base[tid] = valid ? ((long long)kx * g.My + ky) * nl3 : -1;
   __syncthreads();
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   V* __restrict__ Y = pp.work2[blockIdx.y];
   for (int e = tid; e < C4 * nl3; e += C4) {   // all loads in flight at once
     const int cell = by_nl3(e), l = e - cell * nl3;
@@ -461,7 +457,6 @@ __global__ void __launch_bounds__(4 * kBzCells, MZ <= 12 || MZ == 16 || NZ == 11
 template <typename V, int MZ, int NZ>
 __global__ void __launch_bounds__(kBzThreads)
     pass_bz_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g, int tiles, const V* __restrict__ twzg) {
-  if (skip_problem(pp)) return;
   constexpr int C4 = 4 * kBzCells;
   constexpr int KZ = MZ / 2 + 1;
   const int nz = NZ > 0 ? NZ : g.nz, nl3 = 3 * nz;
@@ -502,7 +497,7 @@ __global__ void __launch_bounds__(kBzThreads)
     flip[tid] = (kx > g.Mx - kx ? 1 : 0) | (ky > g.My - ky ? 2 : 0);
   }
   __syncthreads();
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   V* __restrict__ Y = pp.work2[blockIdx.y];
   for (int e = tid; e < C4 * nl3; e += nth) {   // all loads in flight at once
     const int cell = e / nl3, l = e - cell * nl3;
@@ -631,7 +626,6 @@ static vie_status dispatch_pass_bz(const PassPtrs<V>& pp, int count, const PassB
 template <typename V, int MY, int MZ>
 __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__ PassPtrs<V> pp, PassBGeom g,
                                                          const V* __restrict__ twyg, const V* __restrict__ twzg) {
-  if (skip_problem(pp)) return;
   V* __restrict__ work = pp.work[blockIdx.y];
   const V* __restrict__ ghat = pp.ghat[blockIdx.y];
   constexpr int PY = (MY % 2 == 0) ? MY + 1 : MY;
@@ -659,7 +653,7 @@ __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__
     for (int i = tid; i < chunk; i += nth) __pipeline_memcpy_async(Gs + i, G + i, sizeof(V));
     __pipeline_commit();
   }
-  pdl_wait();                 // the x pass that wrote the slab has completed
+  if (skip_after_wait(pp)) return;   // the x pass that wrote the slab has completed
   __pipeline_wait_prior(1);   // twiddles done; the spectrum may still be in flight
   __syncthreads();
   V* slab = work + (size_t)kx * g.NL;
@@ -788,8 +782,7 @@ template <typename V>
 __global__ void __launch_bounds__(256) pass_c_kernel(const __grid_constant__ PassPtrs<V> pp, int nx, int nyz,
                                                      int NL, Radices rx, const V* __restrict__ twg,
                                                      int lines_per_block, int mode, int gsz) {
-  if (skip_problem(pp)) return;
-  pdl_wait();
+  if (skip_after_wait(pp)) return;
   const V* __restrict__ work = pp.work[blockIdx.y];
   const V* __restrict__ x = pp.x[blockIdx.y];
   const V* __restrict__ Mc = pp.M[blockIdx.y];
@@ -845,7 +838,6 @@ __host__ __device__ constexpr int pitch_mod16(int n, int lpb) { return n + ((lpb
 template <typename V, int L1, int L2, int LPB, int NX>
 __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_a4_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int NL, const V* __restrict__ twxg, int gsz) {
-  if (skip_problem(pp)) return;
   static_assert(NX % L1 == 0 && NX % L2 == 0, "compiled line length must divide by L1 and L2");
   const V* __restrict__ x = pp.x[blockIdx.y];
   V* __restrict__ work = pp.work[blockIdx.y];
@@ -866,7 +858,7 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_a4_kernel(
     // asynchronous copies of the twiddles (plan constants) and, once the
     // producer of x is done, of the block's lines (contiguous in x)
     for (int i = tid; i < MX; i += nth) __pipeline_memcpy_async(twx + i, twxg + i, sizeof(V));
-    pdl_wait();
+    if (skip_after_wait(pp)) return;
     const V* src = x + (size_t)l0 * nx;
     for (int l = 0; l < nl; ++l)
       for (int n = tid; n < nx; n += nth) __pipeline_memcpy_async(Xs + l * P + n, src + (size_t)l * nx + n, sizeof(V));
@@ -910,7 +902,6 @@ template <typename V, int L1, int L2, int LPB, int NX>
 __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int nyz, int NL, const V* __restrict__ twxg, int mode,
     int gsz) {
-  if (skip_problem(pp)) return;
   const V* __restrict__ work = pp.work[blockIdx.y];
   const V* __restrict__ x = pp.x[blockIdx.y];
   const V* __restrict__ Mc = pp.M[blockIdx.y];
@@ -939,7 +930,7 @@ __global__ void __launch_bounds__(LPB * (L1 > L2 ? L1 : L2)) pass_c4_kernel(
       const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
       for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
     }
-    pdl_wait();
+    if (skip_after_wait(pp)) return;
     const V* xsrc = x + (size_t)l0 * nx;
     for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
     __pipeline_commit();
@@ -1054,7 +1045,6 @@ __device__ __forceinline__ void x3_steps12(V* __restrict__ S1, V* __restrict__ S
 template <typename V, int L1, int L2, int L3, int LPB, int NX>
 __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_a3_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int NL, const V* __restrict__ twxg, int gsz) {
-  if (skip_problem(pp)) return;
   typedef X3<L1, L2, L3> G;
   static_assert(NX % (L1 * L2) == 0, "compiled line length must divide by L1 L2");
   const V* __restrict__ x = pp.x[blockIdx.y];
@@ -1076,7 +1066,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_a3_kernel(
   pdl_launch_dependents();
   {
     for (int i = tid; i < G::MX; i += nth) __pipeline_memcpy_async(twx + i, twxg + i, sizeof(V));
-    pdl_wait();
+    if (skip_after_wait(pp)) return;
     const V* src = x + (size_t)l0 * nx;
     for (int l = 0; l < nl; ++l)
       for (int n = tid; n < nx; n += nth) __pipeline_memcpy_async(Xs + l * P + n, src + (size_t)l * nx + n, sizeof(V));
@@ -1120,7 +1110,6 @@ template <typename V, int L1, int L2, int L3, int LPB, int NX>
 __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
     const __grid_constant__ PassPtrs<V> pp, int nx, int nyz, int NL, const V* __restrict__ twxg, int mode,
     int gsz) {
-  if (skip_problem(pp)) return;
   typedef X3<L1, L2, L3> G;
   static_assert(NX % G::M == 0, "compiled line length must divide by L2 L3");
   const V* __restrict__ work = pp.work[blockIdx.y];
@@ -1151,7 +1140,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
       const V* msrc = Mc + (size_t)((l0 + l) % nyz) * nx;
       for (int i = tid; i < nx; i += nth) __pipeline_memcpy_async(Ms + l * nx + i, msrc + i, sizeof(V));
     }
-    pdl_wait();
+    if (skip_after_wait(pp)) return;
     const V* xsrc = x + (size_t)l0 * nx;
     for (int e = tid; e < nl * nx; e += nth) __pipeline_memcpy_async(Xs + e, xsrc + e, sizeof(V));
     __pipeline_commit();

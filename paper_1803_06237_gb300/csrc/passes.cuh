@@ -3,6 +3,8 @@
 // the passes for sizes without a compiled kernel of their own.
 #pragma once
 
+#include <cuda_pipeline.h>
+
 #include "vie_internal.cuh"
 
 namespace vie {
@@ -25,12 +27,22 @@ struct PassPtrs {
   const int* live[kMaxBatch]; // per problem: null, or a device flag; 0 skips the problem (its blocks return)
 };
 
-// A problem whose live flag is 0 is skipped by every block of every pass
-// (blockIdx.y is the problem in all grouped launches).
+// The wait for the kernel before, then whether the problem is skipped: one
+// whose live flag is 0 is, by every block of every pass (blockIdx.y is the
+// problem in all grouped launches).  Every pass waits, skipped or not, and
+// reads the flag behind its wait.  A grid whose blocks leave without waiting
+// can complete before the one it was launched behind does; a kernel after it
+// that waits for it alone would then read vectors still being written (several
+// shapes in one call, the last of them skipped).  The copies of plan data that
+// a pass starts ahead of the wait have landed before its blocks leave.
 template <typename V>
-__device__ __forceinline__ bool skip_problem(const PassPtrs<V>& pp) {
+__device__ __forceinline__ bool skip_after_wait(const PassPtrs<V>& pp) {
+  pdl_wait();
   const int* f = pp.live[blockIdx.y];
-  return f != nullptr && *(const volatile int*)f == 0;
+  if (f == nullptr || *(const volatile int*)f != 0) return false;
+  __pipeline_commit();
+  __pipeline_wait_prior(0);
+  return true;
 }
 
 struct PassBGeom {
