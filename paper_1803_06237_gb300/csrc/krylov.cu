@@ -378,10 +378,13 @@ __global__ void __launch_bounds__(kThreads) init_cycle_kernel(const ProbK* __res
   }
 }
 
-// V_0 = r / beta  (converted to the inner type)
+// V_0 = r / beta  (converted to the inner type).  Every cycle begins here, so
+// the barriers' arrival counter starts again too: ticket_barrier's only grows,
+// by a few hundred a barrier, and would wrap in a solve of millions of steps.
 template <typename V>
-__global__ void __launch_bounds__(kThreads) start_vector_kernel(const ProbK* __restrict__ P) {
+__global__ void __launch_bounds__(kThreads) start_vector_kernel(const ProbK* __restrict__ P, unsigned* bar) {
   const ProbK& q = P[blockIdx.y];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *bar = 0u;
   if (!q.st->active) return;
   const double s = q.st->inv_h;
   V* __restrict__ v0 = (V*)q.V;
@@ -1078,29 +1081,29 @@ __global__ void __launch_bounds__(coop_threads<V>(), 1) arnoldi_coop_kernel(cons
 // and write v_{j+1}.  600 x 23 x 11, restart 30: a solve 193 -> 104 ms, 82 us a
 // step of which the operator takes 32 and the basis sweeps about 25.
 //
-// Barrier: a counter that only grows.  A block's ticket t belongs to barrier
-// t / nblocks, which is complete when the counter reaches the next multiple
-// of nblocks.  The wait is bounded by the abort word as in grid_barrier.
-__device__ __forceinline__ bool ticket_barrier(unsigned* bar, unsigned nblocks) {
+// Barrier: a counter that only grows within a cycle (bar[0]; start_vector_kernel
+// clears it).  A block's ticket t belongs to barrier t / nblocks, which is
+// complete when the counter reaches the next multiple of nblocks.  Bounded as
+// grid_barrier: a block that has waited `limit` clocks sets the abort word
+// bar[2], and the others, which look at it every 32nd poll, leave with it.
+__device__ __forceinline__ bool ticket_barrier(unsigned* bar, unsigned nblocks, long long limit = kBarrierCycles) {
   __shared__ int ok_s;
   __syncthreads();
   if (threadIdx.x == 0) {
+    volatile unsigned* vabort = bar + 2;
     __threadfence();
     const unsigned t = atomicAdd(bar, 1u);
     const unsigned target = (t / nblocks + 1u) * nblocks;
     int ok = 1;
     unsigned seen;
     const long long t0 = clock64();
-    while (true) {
+    for (int polls = 1;; ++polls) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
       if ((int)(seen - target) >= 0) break;
-      if (clock64() - t0 > kBarrierCycles) {
-        atomicExch(bar + 2, 1u);
-        ok = 0;
-        break;
-      }
+      if ((polls & 31) == 0 && *vabort) { ok = 0; break; }
+      if (clock64() - t0 > limit) { atomicExch(bar + 2, 1u); ok = 0; break; }
     }
-    ok_s = ok && *(volatile unsigned*)(bar + 2) == 0u;
+    ok_s = ok && !*vabort;
   }
   __syncthreads();
   return ok_s != 0;
@@ -1983,7 +1986,7 @@ static vie_status build_cycle_graph(BatchCall& c, CycleGraph& G, const std::vect
     VIE_CUDA_TRY(cudaStreamBeginCaptureToGraph(G.cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     vie_status st = VIE_OK;
     if (k == 0) {
-      start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, G.cap>>>(c.table);
+      start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, G.cap>>>(c.table, c.bar);
     } else if (k < nodes - 1) {
       const int j0 = (k - 1) * per, j1 = j0 + per < jmax ? j0 + per : jmax;
       for (int j = j0; j < j1 && st == VIE_OK; ++j) {
@@ -2053,7 +2056,7 @@ static vie_status run_cycle(BatchCall& c, CycleGraph& G, const std::vector<int>&
     }
   }
   c.last_cycle_graph = false;
-  start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, s>>>(c.table);
+  start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, s>>>(c.table, c.bar);
   VIE_LAUNCH_CHECK();
   std::vector<int> live = list;       // problems still iterating in this cycle
   for (int j = 0; j < jmax && !live.empty(); ++j) {
@@ -2199,7 +2202,7 @@ static vie_status build_resident_graph(BatchCall& c, ResidentGraph& R, const std
   st = add_segment(B_in, &pi, R.cap, [&](cudaStream_t cs) -> vie_status {
     init_cycle_kernel<<<P, kThreads, 0, cs>>>(c.table, kDotBlocks, m);
     reset_steps_kernel<<<1, 256, 0, cs>>>(R.steps_dev, jmax);
-    start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, cs>>>(c.table);
+    start_vector_kernel<V><<<dim3(gx, P), kThreads, 0, cs>>>(c.table, c.bar);
     VIE_LAUNCH_CHECK();
     return VIE_OK;
   });
@@ -2699,12 +2702,17 @@ extern "C" vie_status vie_jm_solve(vie_plan* p, const void* b, void* x, double t
 }
 
 namespace vie {
-// One grid barrier of the cooperative step in which block `absent` does not
-// take part (it returns first): the other blocks' waits run out after
-// `limit` clocks and set the abort word.
+// Two grid barriers of a cooperative step (TICKET: of the one-problem step), in
+// which block `absent` does not take part (it returns first): the wait of the
+// first of the other blocks runs out after `limit` clocks and sets the abort
+// word, the rest wait without a limit of their own in this test's time and
+// leave by that word.
+template <bool TICKET>
 __global__ void barrier_probe_kernel(unsigned* bar, int absent, long long limit) {
   if ((int)blockIdx.x == absent) return;
-  grid_barrier(bar, gridDim.x, limit);
+  const long long mine = blockIdx.x == (absent == 0 ? 1u : 0u) ? limit : kBarrierCycles;
+  for (int k = 0; k < 2; ++k)
+    if (!(TICKET ? ticket_barrier(bar, gridDim.x, mine) : grid_barrier(bar, gridDim.x, mine))) return;
 }
 }  // namespace vie
 
@@ -2730,7 +2738,6 @@ extern "C" vie_status vie_probe_grid_barrier(int absent_block, double wait_ms, i
   }
   unsigned* bar = nullptr;
   VIE_CUDA_TRY(cudaMalloc((void**)&bar, 4 * sizeof(unsigned)));
-  cudaMemset(bar, 0, 4 * sizeof(unsigned));
   const long long limit = (long long)(wait_ms * (double)clk_khz);   // clk_khz clocks per ms
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)sms);
@@ -2740,14 +2747,23 @@ extern "C" vie_status vie_probe_grid_barrier(int absent_block, double wait_ms, i
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, barrier_probe_kernel, bar, absent_block, limit);
-  unsigned h = 0;
-  if (e == cudaSuccess) e = cudaMemcpy(&h, bar + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
+  unsigned h[2] = {0, 0};   // abort words of the two barriers
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+    e = cudaMemset(bar, 0, 4 * sizeof(unsigned));
+    if (e == cudaSuccess)
+      e = cudaLaunchKernelEx(&cfg, k ? barrier_probe_kernel<true> : barrier_probe_kernel<false>, bar, absent_block, limit);
+    if (e == cudaSuccess) e = cudaMemcpy(&h[k], bar + 2, sizeof(unsigned), cudaMemcpyDeviceToHost);
+  }
   cudaFree(bar);
   if (e != cudaSuccess) {
     set_error("barrier probe: %s", cudaGetErrorString(e));
     return VIE_ERR_CUDA;
   }
-  *aborted = h ? 1 : 0;
+  if (!h[0] != !h[1]) {
+    set_error("the two barriers disagree: abort words %u and %u", h[0], h[1]);
+    return VIE_ERR_TIMEOUT;
+  }
+  *aborted = h[0] ? 1 : 0;
   return VIE_OK;
 }
