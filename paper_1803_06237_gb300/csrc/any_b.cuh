@@ -380,8 +380,7 @@ static vie_status launch_b_any_nc(const PassPtrs<V>& pp, int count, const PassBG
   const dim3 grid((unsigned)g.Mx, (unsigned)count);
   const bool small = g.Mz <= 24 && q.r1 <= 10 && q.r2 <= 6;
   auto run = [&](auto kernel, int threads) -> vie_status {
-    if (smem > 48 * 1024)
-      VIE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(kernel, smem));
     VIE_CUDA_TRY(launch_pdl_if(b_starts_early<V>(g, count), kernel, grid, dim3(threads), smem, s, pp, chat, kappa, g, q, twy));
     return VIE_OK;
   };

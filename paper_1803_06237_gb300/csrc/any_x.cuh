@@ -297,12 +297,10 @@ static vie_status launch_x_any_top(bool forward, const PassPtrs<V>& pp, int coun
   const int threads = ((items + turns - 1) / turns + 31) / 32 * 32;
   const dim3 blocks((unsigned)((NL + g.lpb - 1) / g.lpb), (unsigned)count);
   if (forward) {
-    if (smem > 48 * 1024)
-      VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a_any_kernel<V, TOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_a_any_kernel<V, TOP>, smem));
     VIE_CUDA_TRY(launch_pdl(pass_a_any_kernel<V, TOP>, blocks, dim3(threads), smem, s, pp, g, n, NL, tw, gsz));
   } else {
-    if (smem > 48 * 1024)
-      VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c_any_kernel<V, TOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_c_any_kernel<V, TOP>, smem));
     VIE_CUDA_TRY(launch_pdl(pass_c_any_kernel<V, TOP>, blocks, dim3(threads), smem, s, pp, g, n, nyz, NL, tw, mode, gsz));
   }
   return VIE_OK;

@@ -114,6 +114,7 @@ __device__ __forceinline__ float2 toeplitz_at(const double2* __restrict__ T, int
 // / nx).  tl is chosen so that the 2 tl lines of nx + 1 values fit in shared
 // memory.
 constexpr int kTL = 16;
+constexpr int kBuildShared = kTL * (int)(sizeof(void*) + 4 * sizeof(int));   // static shared memory
 __global__ void __launch_bounds__(256) build_fft_kernel(const double2* __restrict__ T, const float2* __restrict__ Sp,
                                                         const float2* __restrict__ Sm, int nx, int ny, int nz, int tl,
                                                         Radices rd, const float2* __restrict__ twg,
@@ -614,6 +615,7 @@ __device__ __forceinline__ void stream_partial(const float2* __restrict__ A, int
 // that is already final and prefetch block k+1's diagonal block and its
 // coupling block into the other half of double-buffered shared memory.  One
 // barrier per block.  256 threads.
+constexpr int kSolveShared = (2 * 2 * 32 * 33 + 2 * 32 * 8) * (int)sizeof(float2);   // static shared memory
 __global__ void __launch_bounds__(256, 4) circ_solve_kernel(const float2* __restrict__ W, const int* __restrict__ perm,
                                                          float2* __restrict__ vh, int R) {
   extern __shared__ float2 x[];
@@ -931,7 +933,7 @@ static vie_status circ_build(vie_circulant* c, cudaStream_t s, size_t smem_max) 
   // W_hat: blocks formed and transformed along x in shared memory
   const int tl = build_lines(nx, smem_max);
   const size_t fft_smem = (size_t)nx * sizeof(float2) + (size_t)2 * tl * (nx + 1) * sizeof(float2);
-  CIRC_TRY(cudaFuncSetAttribute(build_fft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem));
+  CIRC_TRY(allow_shared(build_fft_kernel, fft_smem, kBuildShared));
   build_fft_kernel<<<(unsigned)((RR + tl - 1) / tl), 256, fft_smem, s>>>(p->toeplitz, Sp, Sm, nx, ny, nz, tl, c->rd,
                                                                         c->tw, c->W);
   CIRC_TRY(cudaGetLastError());
@@ -997,20 +999,19 @@ vie_status circulant_apply(vie_circulant* c, int dtype, const void* v, void* z, 
     zout = c->z32;
   }
   const size_t fft_smem = (size_t)nx * sizeof(float2) + (size_t)2 * kLines * (nx + 1) * sizeof(float2);
-  VIE_CUDA_TRY(cudaFuncSetAttribute(lines_fft_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem));
-  VIE_CUDA_TRY(cudaFuncSetAttribute(lines_fft_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem));
+  VIE_CUDA_TRY(allow_shared(lines_fft_kernel<false>, fft_smem));
+  VIE_CUDA_TRY(allow_shared(lines_fft_kernel<true>, fft_smem));
   // V_hat[w][r] = sum_x exp(-2 pi i w x / nx) v[r][x]
   lines_fft_kernel<false><<<(R + kLines - 1) / kLines, 256, fft_smem, s>>>(vin, c->vh, R, nx, c->rd, c->tw);
   VIE_LAUNCH_CHECK();
   if (c->fp16) {
     const int nb = (R + kTile - 1) / kTile;
     const size_t smem = (size_t)kSolveStages * kStageTiles * kTileElems * sizeof(__half2) + (size_t)nb * kTile * sizeof(float2);
-    VIE_CUDA_TRY(cudaFuncSetAttribute(circ_solve_tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(circ_solve_tiles_kernel, smem, 2 * kTile * sizeof(float)));
     circ_solve_tiles_kernel<<<nx, 256, smem, s>>>(c->W16, c->perm, c->vh, R, nb);
   } else {
-    // the vector and 37 KB of tiles: past 48 KB from 1408 unknowns on
-    VIE_CUDA_TRY(cudaFuncSetAttribute(circ_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(R * sizeof(float2))));
+    // the vector and 37 KB of tiles: past 48 KB from 1409 unknowns on
+    VIE_CUDA_TRY(allow_shared(circ_solve_kernel, R * sizeof(float2), kSolveShared));
     circ_solve_kernel<<<nx, 256, (size_t)R * sizeof(float2), s>>>(c->W, c->perm, c->vh, R);
   }
   VIE_LAUNCH_CHECK();

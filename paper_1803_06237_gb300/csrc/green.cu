@@ -699,7 +699,7 @@ static vie_status launch_spectrum_axis(const double2* in, double2* out, double2*
   int tl = 16;
   while (tl > 1 && tw_bytes + (size_t)tl * per_line > 100 * 1024) tl >>= 1;
   const size_t smem = tw_bytes + (size_t)tl * per_line;
-  VIE_CUDA_TRY(cudaFuncSetAttribute(spectrum_axis_kernel<AXIS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VIE_CUDA_TRY(allow_shared(spectrum_axis_kernel<AXIS>, smem));
   const long long blocks = groups * ((per + tl - 1) / tl);
   spectrum_axis_kernel<AXIS><<<(unsigned)blocks, 256, smem, s>>>(in, out, g64, g32, g, radices_of(ax), ax.tw64, tl,
                                                                scale_);

@@ -309,7 +309,7 @@ static vie_status launch_pass_b_cluster(const PassPtrs<V>& pp, int count, const 
     return VIE_ERR_INVALID;
   }
   const size_t smem = pass_b_cluster_smem(g, q, sizeof(V));
-  VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_cluster_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VIE_CUDA_TRY(allow_shared(pass_b_cluster_kernel<V>, smem));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(g.Mx * q.cs), (unsigned)count);
   cfg.blockDim = dim3(256);
@@ -590,15 +590,13 @@ static vie_status launch_pass_bz(const PassPtrs<V>& pp, int count, const PassBGe
   const dim3 grid((unsigned)((g.Mx / 2 + 1) * tiles), (unsigned)count);
   if constexpr (sizeof(V) == sizeof(float2)) {
     const size_t smem = C4 * sizeof(long long) + (spec + (size_t)C4 * pio) * sizeof(V);
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_bz_cells_kernel<MZ, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_bz_cells_kernel<MZ, NZ>, smem));
     VIE_CUDA_TRY(launch_pdl(pass_bz_cells_kernel<MZ, NZ>, grid, dim3(C4), smem, s, pp, g, tiles,
                             (unsigned)((0x100000000ull + nl3 - 1) / nl3)));
   } else {
     const size_t smem = (size_t)C4 * (sizeof(long long) + sizeof(int)) + (MZ + spec + 3 * MZ * C4) * sizeof(V);
     if (smem > 220 * 1024) { set_error("pass B2 shared memory %zu too large", smem); return VIE_ERR_INVALID; }
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_bz_kernel<V, MZ, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_bz_kernel<V, MZ, NZ>, smem));
     VIE_CUDA_TRY(launch_pdl(pass_bz_kernel<V, MZ, NZ>, grid, dim3(kBzThreads), smem, s, pp, g, tiles, twz));
   }
   return VIE_OK;
@@ -740,8 +738,7 @@ static vie_status launch_pass_b_reg(const PassPtrs<V>& pp, int count, const Pass
   constexpr int PZ = (MZ % 2 == 0) ? MZ + 1 : MZ;
   const size_t smem = (size_t)(MY + MZ + 3 * MZ * PY + 3 * g.ny * PZ + 6 * g.Kz * g.Ky) * sizeof(V);
   if (smem > 220 * 1024) { set_error("pass B shared memory %zu too large", smem); return VIE_ERR_INVALID; }
-  VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_reg_kernel<V, MY, MZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+  VIE_CUDA_TRY(allow_shared(pass_b_reg_kernel<V, MY, MZ>, smem));
   int lines = 3 * (g.ny > MZ ? g.ny : MZ);
   int threads = ((lines + 31) / 32) * 32;
   if (threads > 256) threads = 256;
@@ -1195,7 +1192,7 @@ __global__ void __launch_bounds__(LPB * X3<L1, L2, L3>::NT) pass_c3_kernel(
 // 13; at every other size those are the faster ones.
 template <typename V, typename Kernel, typename... Args>
 static vie_status launch_x_lines(Kernel kernel, dim3 blocks, int threads, size_t smem, cudaStream_t s, Args... args) {
-  VIE_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VIE_CUDA_TRY(allow_shared(kernel, smem));
   VIE_CUDA_TRY(launch_pdl(kernel, blocks, dim3(threads), smem, s, args...));
   return VIE_OK;
 }
@@ -1279,10 +1276,10 @@ static vie_status launch_x_generic(bool forward, const PassPtrs<V>& pp, int coun
   }
   const dim3 blocks((unsigned)((NL + lpb - 1) / lpb), (unsigned)count);
   if (forward) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_a_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_a_kernel<V>, smem));
     pass_a_kernel<V><<<blocks, 256, smem, s>>>(pp, n, NL, rd, tw, lpb, gsz);
   } else {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_c_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA_TRY(allow_shared(pass_c_kernel<V>, smem));
     pass_c_kernel<V><<<blocks, 256, smem, s>>>(pp, n, nyz, NL, rd, tw, lpb, mode, gsz);
   }
   VIE_LAUNCH_CHECK();
@@ -1347,7 +1344,7 @@ static vie_status run_passes(const vie_plan* p, const PassPtrs<V>& pp, int count
     done = true;
   }
   if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
+    VIE_CUDA_TRY(allow_shared(pass_b_kernel<V>, smem_b));
     pass_b_kernel<V><<<dim3((unsigned)Mx, (unsigned)count), threads, smem_b, s>>>(pp, g, radices_of(p->ax[1]),
                                                                                 radices_of(p->ax[2]), twy, twz);
     VIE_LAUNCH_CHECK();
@@ -1633,15 +1630,14 @@ static vie_status run_jm(vie_plan* p, const V* x, V* y, const V* ghat, const V* 
     if (st != VIE_OK) return st;
   }
   if (!done && smem_b <= 220 * 1024) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_jm_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
+    VIE_CUDA_TRY(allow_shared(pass_b_jm_kernel<V>, smem_b));
     pass_b_jm_kernel<V><<<(unsigned)Mx, 256, smem_b, s>>>((V*)p->jm_work, ghat, chat, g, radices_of(p->ax[1]),
                                                           radices_of(p->ax[2]), twy, twz, p->kappa);
     VIE_LAUNCH_CHECK();
     done = true;
   }
   if (!done) {
-    VIE_CUDA_TRY(cudaFuncSetAttribute(pass_b_jm_lines_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem_bl));
+    VIE_CUDA_TRY(allow_shared(pass_b_jm_lines_kernel<V>, smem_bl));
     pass_b_jm_lines_kernel<V><<<(unsigned)Mx, 256, smem_bl, s>>>((V*)p->jm_work, ghat, chat, g,
                                                                  radices_of(p->ax[1]), radices_of(p->ax[2]), twy,
                                                                  twz, p->kappa);

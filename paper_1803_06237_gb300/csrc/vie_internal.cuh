@@ -85,6 +85,19 @@ template <typename V> __host__ __device__ __forceinline__ V mul_pi(V a) { V r; r
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
+// Lets a launch take `smem` bytes of dynamic shared memory past 48 KB.  The limit
+// is state of the kernel, not of the launch: it is always set to the same
+// value, all that a block can have beside the kernel's `fixed` bytes of static
+// shared memory.  Set to the size of each call, a smaller call on another host
+// thread could lower it between this one's setting and its launch, which was
+// then refused (one kernel serves plans of many sizes).
+constexpr int kMaxShared = 227 * 1024;
+template <typename... KArgs>
+static inline cudaError_t allow_shared(void (*kernel)(KArgs...), size_t smem, int fixed = 0) {
+  if (smem + fixed <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxShared - fixed);
+}
+
 // Launch with programmatic stream serialisation, if `early`.
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_pdl_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
