@@ -61,9 +61,11 @@ struct DwLayer {
   int nxp, nxc;              // padded row, chunks per row
   int block0;                // first block of the operand launch
   int cta0, ctas;            // CTAs of the GEMM
+  int layer;                 // its maps
 };
 struct DwArgs {
-  DwLayer l[kNumLayers];
+  DwLayer l[kNumLayers];     // the `count` layers of this group
+  int count;
   int stages;
   float* partial;            // [CTA][27][32][C], CTAs 27 x 32 x 32 apart
   int* bad;
@@ -80,7 +82,7 @@ struct DwArgs {
 __global__ void __launch_bounds__(256) dw_operands_kernel(const __grid_constant__ DwArgs args) {
   __shared__ __nv_bfloat16 t[kDwChunk + 2][33];
   __shared__ float bsum[8][33];
-  int li = kNumLayers - 1;
+  int li = args.count - 1;
   while (li > 0 && (int)blockIdx.x < args.l[li].block0) --li;
   const DwLayer& L = args.l[li];
   const Dims d = L.d;
@@ -258,13 +260,13 @@ constexpr size_t kDwPartial = (size_t)27 * 32 * 32;   // floats of a CTA's parti
 
 __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_constant__ DwMaps maps,
                                                               const __grid_constant__ DwArgs args) {
-  int li = kNumLayers - 1;
+  int li = args.count - 1;
   while (li > 0 && (int)blockIdx.x < args.l[li].cta0) --li;
   const DwLayer& L = args.l[li];
   const int cta = blockIdx.x - L.cta0;
   float* partial = args.partial + blockIdx.x * kDwPartial;
-  if (L.C == 32) dw_gemm<32>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
-  else dw_gemm<16>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
+  if (L.C == 32) dw_gemm<32>(maps.a[L.layer], maps.b[L.layer], L, cta, args.stages, partial, args.bad);
+  else dw_gemm<16>(maps.a[L.layer], maps.b[L.layer], L, cta, args.stages, partial, args.bad);
 }
 
 // gw[(o ci + c) 27 + t] += sum_b partial[b][t][o][c] over the layer's CTAs
@@ -442,6 +444,7 @@ struct TcTrain {
   __nv_bfloat16 *dY = nullptr, *dpre[kNumLayers] = {}, *ddecin[3] = {}, *da[4] = {};
   __nv_bfloat16 *Apl[kNumLayers] = {}, *Bpl[kNumLayers] = {};   // planar GEMM operands of each layer
   size_t plane[kNumLayers] = {};                                // their row strides (elements)
+  int group[kNumLayers] = {};                                   // layers whose operands are there together
   float* Yf = nullptr;                             // network output [V0][16]
   size_t yf_cap = 0;
   float* partial = nullptr;                        // [sms] partial sums of kDwPartial
@@ -458,6 +461,15 @@ struct TcTrain {
 
 constexpr size_t kMapAlign = 128;   // elements: operand buffers start on 256 bytes
 
+// Most memory for the planar operands (elements, 1 GiB), past which the layers
+// take turns with it: all of them together are 1130 bytes a voxel (rows padded
+// to 64), the largest layer's 320, everything else of a sample 850.
+// Consecutive layers share a group of launches while they fit the larger of
+// this and one layer.  One group against four: 326 against 401 us a sample on
+// 160 x 40 x 11, 1063 against 1132 on 400 x 100 x 11, no difference from a
+// million voxels on (960 x 160 x 12: 3.59 ms), where the line lies.
+constexpr size_t kDwOperands = (size_t)1 << 29;
+
 static int nxp_of(int nx) { return (nx + kDwChunk - 1) / kDwChunk * kDwChunk; }
 
 void tc_train_free(TcTrain* t) {
@@ -469,7 +481,7 @@ void tc_train_free(TcTrain* t) {
   delete t;
 }
 
-static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const int n[3]) {
+static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const int n[3], cudaStream_t s) {
   if (!*pt) *pt = new TcTrain();
   TcTrain* T = *pt;
   // keyed on the buffers, so that a failed allocation is retried next time
@@ -499,11 +511,16 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
     for (int l = 1; l < 4; ++l) need += 32 * T->L[l].vox();       // a_l
     for (int l = 0; l < 3; ++l) need += 32 * T->L[l].vox() * 3;   // decin_l, u_l, ddecin_l
     for (int l = 0; l < kNumLayers; ++l) need += 32 * T->L[kLayerLevel[l]].vox();   // dpre
-    for (int l = 0; l < kNumLayers; ++l) {                        // Apl, Bpl
+    size_t opnd[kNumLayers], all = 0, most = 0;                   // Apl, Bpl
+    for (int l = 0; l < kNumLayers; ++l) {
       const Dims d = T->L[kLayerLevel[l]];
       T->plane[l] = (size_t)d.nz * d.ny * nxp_of(d.nx);
-      need += (128 + tc_cpad(kLayerDefs[l].ci)) * T->plane[l] + 2 * kMapAlign;
+      opnd[l] = ((128 + tc_cpad(kLayerDefs[l].ci)) * T->plane[l] + kMapAlign - 1) / kMapAlign * kMapAlign;
+      all += opnd[l];
+      if (opnd[l] > most) most = opnd[l];
     }
+    const size_t operands = all <= kDwOperands ? all : most > kDwOperands ? most : kDwOperands;
+    need += operands + kMapAlign;
     if (need > T->cap) {
       cudaFree(T->ws);
       T->ws = nullptr;
@@ -537,13 +554,18 @@ static vie_status tc_train_prepare(TcTrain** pt, const TcTrainParams& P, const i
       T->ddecin[l] = take(32 * T->L[l].vox());
     }
     for (int l = 0; l < kNumLayers; ++l) T->dpre[l] = take(32 * T->L[kLayerLevel[l]].vox());
-    for (int l = 0; l < kNumLayers; ++l) {
-      p = T->ws + ((p - T->ws) + kMapAlign - 1) / kMapAlign * kMapAlign;
-      T->Apl[l] = take(128 * T->plane[l]);
-      T->Bpl[l] = take(tc_cpad(kLayerDefs[l].ci) * T->plane[l]);
-      // rows 96..127 of A (no dx block) stay zero
-      VIE_CUDA_TRY(cudaMemset(T->Apl[l] + 96 * T->plane[l], 0, 32 * T->plane[l] * sizeof(__nv_bfloat16)));
+    p = T->ws + ((p - T->ws) + kMapAlign - 1) / kMapAlign * kMapAlign;
+    size_t at = 0;
+    for (int l = 0, g = 0; l < kNumLayers; ++l) {
+      if (at + opnd[l] > operands) { ++g; at = 0; }
+      T->group[l] = g;
+      T->Apl[l] = p + at;
+      T->Bpl[l] = T->Apl[l] + 128 * T->plane[l];
+      at += opnd[l];
     }
+    // rows 96..127 of A (no dx block) are never written; their accumulators are
+    // never read
+    VIE_CUDA_TRY(cudaMemsetAsync(p, 0, operands * sizeof(__nv_bfloat16), s));
     // forward maps: the inputs of enc0..enc3, dec2, dec1, dec0, out
     const __nv_bfloat16* in[kNumLayers] = {T->X, T->a[1], T->a[2], T->a[3], T->decin[2], T->decin[1], T->decin[0],
                                            T->u[0]};
@@ -587,16 +609,19 @@ static unsigned ew_grid(size_t n) {
   return (unsigned)(b < 152 * 16 ? (b ? b : 1) : 152 * 16);
 }
 
-// Weight and bias gradients of every layer from its pre-activation gradient
-// (NPo channels) and its input (tc_cpad(ci) channels), added to grad.
-static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, cudaStream_t s) {
+// Weight and bias gradients of the layers l0 .. l1 - 1 from their pre-activation
+// gradients (NPo channels) and inputs (tc_cpad(ci) channels), added to grad.
+static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, int l0, int l1, cudaStream_t s) {
   const __nv_bfloat16* in[kNumLayers] = {T->X, T->a[1], T->a[2], T->a[3], T->decin[2], T->decin[1], T->decin[0],
                                          T->u[0]};
   DwArgs a{};
-  long chunks[kNumLayers], total = 0, want = 0;
+  a.count = l1 - l0;
+  long chunks[kNumLayers], want = 0;
   unsigned blocks = 0;
-  for (int l = 0; l < kNumLayers; ++l) {
-    DwLayer& L = a.l[l];
+  for (int k = 0; k < a.count; ++k) {
+    const int l = l0 + k;
+    DwLayer& L = a.l[k];
+    L.layer = l;
     L.d = T->L[kLayerLevel[l]];
     L.g = l == OUTL ? T->dY : T->dpre[l];
     L.in = in[l];
@@ -613,25 +638,24 @@ static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, cuda
     L.nxc = L.nxp / kDwChunk;
     L.block0 = (int)blocks;
     blocks += (unsigned)(2 * L.nxc * L.d.ny * L.d.nz);
-    chunks[l] = (long)L.d.nz * L.d.ny * L.nxc;
-    total += chunks[l];
-    want += (chunks[l] + kDwMinChunks - 1) / kDwMinChunks;
+    chunks[k] = (long)L.d.nz * L.d.ny * L.nxc;
+    want += (chunks[k] + kDwMinChunks - 1) / kDwMinChunks;
   }
   // one CTA per SM at most, each layer's share by its chunks: one each, then
   // to the layer with the most chunks a CTA
   const int ctas = (int)(want < T->sms ? want : T->sms);
-  for (int l = 0; l < kNumLayers; ++l) a.l[l].ctas = 1;
-  for (int k = kNumLayers; k < ctas; ++k) {
+  for (int k = 0; k < a.count; ++k) a.l[k].ctas = 1;
+  for (int n = a.count; n < ctas; ++n) {
     int most = 0;
-    for (int l = 1; l < kNumLayers; ++l)
-      if (chunks[l] * a.l[most].ctas > chunks[most] * a.l[l].ctas) most = l;
+    for (int k = 1; k < a.count; ++k)
+      if (chunks[k] * a.l[most].ctas > chunks[most] * a.l[k].ctas) most = k;
     if (a.l[most].ctas >= chunks[most]) break;
     ++a.l[most].ctas;
   }
   int used = 0;
-  for (int l = 0; l < kNumLayers; ++l) {
-    a.l[l].cta0 = used;
-    used += a.l[l].ctas;
+  for (int k = 0; k < a.count; ++k) {
+    a.l[k].cta0 = used;
+    used += a.l[k].ctas;
   }
   constexpr size_t SB = 128 * 128 + 9 * 32 * 128;
   const size_t fixed = 1024 + 2 * kDwMaxStages * 8 + 64;
@@ -650,14 +674,14 @@ static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, cuda
   VIE_CUDA_TRY(cudaFuncSetAttribute(dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dw_tc_kernel<<<used, kDwThreads, smem, s>>>(T->mP, a);
   VIE_LAUNCH_CHECK();
-  dw_reduce_kernel<<<dim3((unsigned)(kDwPartial / 256), kNumLayers, 8), 256, 0, s>>>(a);
+  dw_reduce_kernel<<<dim3((unsigned)(kDwPartial / 256), (unsigned)a.count, 8), 256, 0, s>>>(a);
   VIE_LAUNCH_CHECK();
   return VIE_OK;
 }
 
 vie_status tc_train_accumulate(TcTrain** pt, const TcTrainParams& P, const int n[3], const double2* chi,
                                const float2* r, const float2* e, double* loss, cudaStream_t s) {
-  vie_status st = tc_train_prepare(pt, P, n);
+  vie_status st = tc_train_prepare(pt, P, n, s);
   if (st != VIE_OK) return st;
   TcTrain* T = *pt;
   const Dims L0 = T->L[0];
@@ -729,7 +753,10 @@ vie_status tc_train_accumulate(TcTrain** pt, const TcTrainParams& P, const int n
                                                                       L[l - 1], T->dpre[ENC0 + l - 1]);
     VIE_LAUNCH_CHECK();
   }
-  if ((st = weight_grads_tc(T, P, s)) != VIE_OK) return st;
+  for (int l = 0, end; l < kNumLayers; l = end) {
+    for (end = l + 1; end < kNumLayers && T->group[end] == T->group[l];) ++end;
+    if ((st = weight_grads_tc(T, P, l, end, s)) != VIE_OK) return st;
+  }
   if (loss) {
     double h[3] = {0, 0, 0};
     VIE_CUDA_TRY(cudaMemcpyAsync(h, sums, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
