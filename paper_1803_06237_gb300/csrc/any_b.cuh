@@ -22,15 +22,46 @@ namespace vie {
 // Place of (c, kz; n1 or k1, n2): (c Mz + kz) py + p2 k1 + n2, p2 = r2 | 1,
 // py = r1 p2: rows of stage items and of fused items fall on distinct banks.
 // ---------------------------------------------------------------------------
-// Sizes known at compile time (the benchmark's 460 x 220 nm strip, 23 x 11
-// voxels in 45 or 48 x 24): the same kernel with its divisions, strides and
-// switches folded.  Zeros: all at run time.
-template <int R1_, int R2_, int MZ_, int NY_, int NZ_, int PY_>
+// Row pitch py = r1 p2 + pad with the fewest bank conflicts of the two patterns
+// that cross rows: stage items (row py + n2) and fused items (kz py + p2 k1).
+// An element is 8 or 16 bytes and a shared-memory phase serves 128, i.e. 16
+// or 8 lanes.  Without it the 54 x 24 planes of the Bragg grating spent half
+// of their shared-memory cycles on conflicts.
+constexpr int b_pad(int r1, int r2, int lanes) {
+  int best = 1 << 30, at = 0;
+  for (int pad = 0; pad < lanes; ++pad) {
+    const int p2 = r2 | 1, py = r1 * p2 + pad;
+    int cost = pad;   // ties: the smaller plane
+    for (int warp = 0; warp < 96; warp += lanes) {
+      int n1[16] = {0}, n2[16] = {0};
+      for (int i = warp; i < warp + lanes; ++i) {
+        ++n1[(i / r2 * py + i % r2) % lanes];
+        ++n2[(i / r1 * py + i % r1 * p2) % lanes];
+      }
+      for (int k = 0; k < lanes; ++k) cost += 16 * (n1[k] * n1[k] + n2[k] * n2[k]);
+    }
+    if (cost < best) { best = cost; at = pad; }
+  }
+  return at;
+}
+
+// Transform lengths known at compile time: the same kernel (complex64) with its
+// divisions by them, its strides and its switches folded; the cross-section
+// stays a run-time value (21 to 24 x 11 or 12 voxels meet in 45 or 48 x 24; with
+// 23 x 11 compiled in too, that one took 30.1 us instead of 30.3 and the others
+// stayed behind by 5 to 20 %).  Zeros: all at run time.
+template <int R1_, int R2_, int MZ_>
 struct BFix {
-  static constexpr int R1 = R1_, R2 = R2_, MZ = MZ_, NY = NY_, NZ = NZ_, PY = PY_, P2 = R2_ | 1;
+  static constexpr int R1 = R1_, R2 = R2_, MZ = MZ_, P2 = R2_ | 1;
   static constexpr bool on = R1_ > 0;
+  // voxels that every cross-section of the plane has: all but the last one of z,
+  // all rows of r2 but the last one of y (taken only where they are there)
+  static constexpr int min_z = MZ_ / 2 - 1, min_y = R2_ * ((R1_ + 1) / 2 - 1);
+  static __device__ __forceinline__ bool full_z(int z) { return on && z < min_z; }
+  static __device__ __forceinline__ bool full_y(int n1) { return on && R2_ * (n1 + 1) <= min_y; }
+  static constexpr int PY = on ? R1_ * P2 + b_pad(on ? R1_ : 1, on ? R2_ : 1, 16) : 0;
 };
-typedef BFix<0, 0, 0, 0, 0, 0> BFree;
+typedef BFix<0, 0, 0> BFree;
 
 #define VIE_Z_LENGTHS(X) \
   X(1) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(12) X(15) X(16) X(18) X(20) X(24) X(25) X(27) X(30) X(32)
@@ -104,11 +135,11 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
   extern __shared__ unsigned char smem_raw[];
   V* S = reinterpret_cast<V*>(smem_raw);
   const int kx = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  const int ny = FIX::on ? FIX::NY : g.ny, nz = FIX::on ? FIX::NZ : g.nz, Mz = FIX::on ? FIX::MZ : g.Mz;
+  const int ny = g.ny, nz = g.nz, Mz = FIX::on ? FIX::MZ : g.Mz;
   const int r1 = FIX::on ? FIX::R1 : q.r1, r2 = FIX::on ? FIX::R2 : q.r2;
   const int p2 = FIX::on ? FIX::P2 : q.p2, py = FIX::on ? FIX::PY : q.py;
   const int My = FIX::on ? FIX::R1 * FIX::R2 : g.My, Ky = FIX::on ? My / 2 + 1 : g.Ky;
-  auto by_ny = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::NY : 1) : div_by(v, q.mny); };
+  auto by_ny = [&](int v) { return FIX::on ? (int)__umulhi((unsigned)v, q.mny) : div_by(v, q.mny); };
   auto by_r1 = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::R1 : 1) : div_by(v, q.mr1); };
   auto by_r2 = [&](int v) { return FIX::on ? v / (FIX::on ? FIX::R2 : 1) : div_by(v, q.mr2); };
   const bool fx = kx > g.Mx - kx;
@@ -135,9 +166,10 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
       for (int it = tid; it < 2 * NC * ny; it += nth) {
         const int line = it >> 1, odd = it & 1;
         const int c = by_ny(line), y = line - c * ny;
+        const V* src = slab + c * nz * ny + y;
         V a[M];
 #pragma unroll
-        for (int z = 0; z < M; ++z) a[z] = z < nz ? slab[(c * nz + z) * ny + y] : zero_c<V>();
+        for (int z = 0; z < M; ++z, src += ny) a[z] = (FIX::full_z(z) || z < nz) ? *src : zero_c<V>();
         if (odd) half_twiddle<V, false, MZ>(a);
         reg_fft<V, false, M>(a, nullptr);
         V* d = S + (c * MZ + odd) * py + y + (p2 - r2) * by_r2(y);
@@ -166,7 +198,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
       V a[R1];
 #pragma unroll
       for (int n1 = 0; n1 < R1; ++n1)
-        a[n1] = (n1 < (R1 + 1) / 2 && n2 + r2 * n1 < ny) ? d[n1 * p2] : zero_c<V>();
+        a[n1] = (n1 < (R1 + 1) / 2 && (FIX::full_y(n1) || n2 + r2 * n1 < ny)) ? d[n1 * p2] : zero_c<V>();
       reg_fft<V, false, R1, (R1 + 1) / 2>(a, nullptr);
 #pragma unroll
       for (int k1 = 0; k1 < R1; ++k1) d[k1 * p2] = a[k1];
@@ -249,7 +281,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
       reg_fft<V, true, R1>(a, nullptr);
 #pragma unroll
       for (int n1 = 0; n1 < (R1 + 1) / 2; ++n1)
-        if (n2 + r2 * n1 < ny) d[n1 * p2] = a[n1];
+        if (FIX::full_y(n1) || n2 + r2 * n1 < ny) d[n1 * p2] = a[n1];
     }
   });
   __syncthreads();
@@ -280,7 +312,7 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
           got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
           const int z = odd ? h + H : h;
           const V mine = odd ? (h + H < M ? a[h + H] : zero_c<V>()) : a[h];
-          if (in && z < nz) o[z * ny] = add(mine, got);
+          if (in && (FIX::full_z(z) || z < nz)) o[z * ny] = add(mine, got);
         }
       }
     } else {
@@ -299,33 +331,14 @@ __global__ void __launch_bounds__(256, sizeof(V) == sizeof(float2) ? (SMALL && N
   });
 }
 
-// Row pitch py >= r1 p2 with the fewest bank conflicts of the two patterns
-// that cross rows: stage items (row py + n2) and fused items (kz py + p2 k1).
-// An element is 8 or 16 bytes and a shared-memory phase serves 128, i.e. 16
-// or 8 lanes.  Without it the 54 x 24 planes of the Bragg grating spent half
-// of their shared-memory cycles on conflicts.
-struct BPitch {
+// b_pad of every split
+struct BPads {
   unsigned char pad[17][11];
 };
-static BPitch b_pitches(int lanes) {
-  BPitch t;
+static BPads b_pads(int lanes) {
+  BPads t;
   for (int r1 = 1; r1 <= 16; ++r1)
-    for (int r2 = 1; r2 <= 10; ++r2) {
-      int best = 1 << 30;
-      for (int pad = 0; pad < lanes; ++pad) {
-        const int p2 = r2 | 1, py = r1 * p2 + pad;
-        int cost = pad;   // ties: the smaller plane
-        for (int warp = 0; warp < 96; warp += lanes) {
-          int n1[16] = {0}, n2[16] = {0};
-          for (int i = warp; i < warp + lanes; ++i) {
-            ++n1[(i / r2 * py + i % r2) % lanes];
-            ++n2[(i / r1 * py + i % r1 * p2) % lanes];
-          }
-          for (int k = 0; k < lanes; ++k) cost += 16 * (n1[k] * n1[k] + n2[k] * n2[k]);
-        }
-        if (cost < best) { best = cost; t.pad[r1][r2] = (unsigned char)pad; }
-      }
-    }
+    for (int r2 = 1; r2 <= 10; ++r2) t.pad[r1][r2] = (unsigned char)b_pad(r1, r2, lanes);
   return t;
 }
 
@@ -333,7 +346,7 @@ static BPitch b_pitches(int lanes) {
 // class (r1 <= 10, r2 <= 6) where possible.
 template <typename V, int NC>
 static bool b_any_split(int ny, int my, BAny* q) {
-  static const BPitch pitch = b_pitches(128 / (int)sizeof(V));
+  static const BPads pads = b_pads(128 / (int)sizeof(V));
   int best = -1;
   const int r1s[] = {
 #define VIE_X(a) a,
@@ -347,7 +360,7 @@ static bool b_any_split(int ny, int my, BAny* q) {
       const int cost = (r1 > r2 ? r1 - r2 : r2 - r1) + (r2 > 6 || r1 > 10 ? 1000 : 0);
       if (best >= 0 && cost >= best) continue;
       best = cost;
-      *q = BAny{r1, r2, r2 | 1, r1 * (r2 | 1) + pitch.pad[r1][r2], div_magic(ny), div_magic(r1), div_magic(r2)};
+      *q = BAny{r1, r2, r2 | 1, r1 * (r2 | 1) + pads.pad[r1][r2], div_magic(ny), div_magic(r1), div_magic(r2)};
     }
   return best >= 0;
 }
@@ -386,19 +399,20 @@ static vie_status launch_b_any_nc(const PassPtrs<V>& pp, int count, const PassBG
   };
   vie_status st;
   if constexpr (sizeof(V) == sizeof(float2)) {
-    // the compiled sizes, where they are what was chosen for this plane (the
-    // shared memory above is laid out with q's radices and pitch)
+    typedef BFix<9, 5, 24> F45;
+    typedef BFix<8, 6, 24> F48;
     auto is = [&](auto fix) {
       typedef decltype(fix) F;
-      return g.ny == F::NY && g.nz == F::NZ && g.Mz == F::MZ && g.My == F::R1 * F::R2 && q.r1 == F::R1 &&
-             q.r2 == F::R2 && q.p2 == F::P2 && q.py == F::PY && g.Ky == g.My / 2 + 1 && g.Kz == g.Mz / 2 + 1;
+      return q.r1 == F::R1 && q.r2 == F::R2 && g.Mz == F::MZ && g.nz >= F::min_z && g.ny >= F::min_y;
     };
-    typedef BFix<9, 5, 24, 23, 11, 45> F45;
-    typedef BFix<8, 6, 24, 23, 11, 70> F48;
     if (stage && (is(F45{}) || is(F48{}))) {
-      // five warps for three components: two turns of the fused phase and three
-      // of the first y stage (600 x 23 x 11: 30.7 us an application against
-      // 31.8 with seven, 33.7 with four warps)
+      // Compiled with their radices these planes take 8 to 20 % less than with
+      // run-time ones (600 x 23 x 11: 30.3 us an application against 34.4; 600 x
+      // 24 x 12: 35.7 against 39.1; 250 x 22 x 12: 19.3 against 24.3; JM 600 x 22 x
+      // 11: 67.9 against 75.9).  Three components: five warps, one turn of the z
+      // phase, two of the fused phase and three of the first y stage (600 x 23 x
+      // 11: 30.5 with five, 32.0 with seven; 250 x 21 x 11: 20.2, 21.3 with seven,
+      // 22.7 with four; 600 x 24 x 12: 35.9, 35.7 with six).
       const int t = NC == 3 ? 160 : threads;
       st = is(F45{}) ? run(pass_b_any_kernel<V, NC, true, true, F45>, t) : run(pass_b_any_kernel<V, NC, true, true, F48>, t);
       if (st != VIE_OK) return st;

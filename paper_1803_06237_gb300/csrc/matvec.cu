@@ -726,10 +726,10 @@ __global__ void __launch_bounds__(256) pass_b_reg_kernel(const __grid_constant__
 }
 
 // (MY, MZ) pairs with this pass B: at these planes it is up to a tenth faster
-// than the kernel with run-time radices (500 x 24 x 13: 34.6 us an application
-// against 38.8), which serves every other size.
+// than the kernel of any_b.cuh (500 x 24 x 13: 34.6 us an application against
+// 38.8), which serves every other size.
 #define VIE_PASS_B_REG_SIZES(X) \
-  X(24, 24) X(45, 24) X(48, 24) X(50, 24) X(30, 24) X(40, 24) X(25, 24) X(45, 25) X(48, 25) X(24, 25)
+  X(24, 24) X(50, 24) X(30, 24) X(40, 24) X(25, 24) X(45, 25) X(48, 25) X(24, 25)
 
 template <typename V, int MY, int MZ>
 static vie_status launch_pass_b_reg(const PassPtrs<V>& pp, int count, const PassBGeom& g, const V* twy,
@@ -766,7 +766,6 @@ static vie_status dispatch_pass_b_reg(const PassPtrs<V>& pp, int count, const Pa
   *done = false;
 #define VIE_X(a, b) \
   if (g.My == a && g.Mz == b) return try_pass_b_reg<V, a, b>(pp, count, g, twy, twz, s, done);
-  if (b_any_compiled(g)) return VIE_OK;   // launch_b_any's kernel for this plane is the faster one
   VIE_PASS_B_REG_SIZES(VIE_X)
 #undef VIE_X
   return VIE_OK;

@@ -1,4 +1,4 @@
-// Shared by the operator's pass kernels (matvec.cu, matvec_any.cu): the
+// Shared by the operator's pass kernels (matvec.cu, any_x.cuh, any_b.cuh): the
 // per-problem pointers of a launch, the plane geometry, and the launchers of
 // the passes for sizes without a compiled kernel of their own.
 #pragma once
@@ -69,13 +69,6 @@ template <typename V> inline bool b_starts_early(const PassBGeom& g, int count) 
 template <typename V>
 vie_status launch_x_any(bool forward, const PassPtrs<V>& pp, int count, int n, int nyz, int NL, int len, const V* tw,
                         int mode, cudaStream_t s, int gsz, bool* done);
-
-// Planes whose sizes are compiled into launch_b_any's complex64 kernel: the
-// 460 x 220 nm strip at 20 nm (23 x 11 voxels) in its smallest 5-smooth
-// embeddings.
-inline bool b_any_compiled(const PassBGeom& g) {
-  return g.ny == 23 && g.nz == 11 && g.Mz == 24 && (g.My == 45 || g.My == 48);
-}
 
 // Pass B on one CTA per kx with run-time radices: nc = 3 (J-VIE) or 6
 // (JM-VIE: pp.work[0], pp.ghat[0], chat and kappa, one problem).  *done =

@@ -88,3 +88,13 @@ def test_compiled_cross_section():
     for dtype, tol in ((np.complex64, 2e-6), (np.complex128, 1e-12)):
         test_operator_and_source((13, 23, 11), dtype, tol)
         test_jm_operator((13, 23, 11), dtype, tol)
+
+
+# the planes whose radices are compiled in (45 x 24 and 48 x 24) with every cross-section that meets in them
+@pytest.mark.parametrize("grid", [(13, 21, 11), (12, 21, 12), (7, 22, 11), (16, 22, 12), (9, 23, 12), (13, 24, 11),
+                                  (20, 24, 12)])
+def test_compiled_planes(grid):
+    from paper_1803_06237_gb300 import vie
+    assert vie.vie_plan_create(grid, 0.02, 4.05, 2.085).info()["m"][1:] == (48 if grid[1] == 24 else 45, 24)
+    test_operator_and_source(grid, np.complex64, 2e-6)
+    test_jm_operator(grid, np.complex64, 2e-6)
