@@ -73,7 +73,9 @@ __device__ __forceinline__ void store_bf16_row(__nv_bfloat16* dst, const float (
 // v + y (hi + lo) to the accuracy of a 64-bit sum, in FP32: Dekker's exact
 // product and Knuth's exact sum.  (The FP64 form held the output layer to two
 // operations a clock; a network application on the 600 x 23 x 11 guide 110.4 ->
-// 106.2 us, the same bits.)
+// 106.2 us, the same bits.)  For scales within 2^+-100: near the ends of the FP32
+// range the product's error term underflows (2 units in the last place at
+// 2^-118) or the product overflows where the sum does not.
 __device__ __forceinline__ float add_scaled(float v, float y, float hi, float lo) {
   const float p = __fmul_rn(y, hi);
   const float e = __fmaf_rn(y, lo, __fmaf_rn(y, hi, -p));
@@ -217,7 +219,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) conv_tc_kernel(const __grid_con
       const double ss = *a.sumsq;
       inv = ss > 0.0 ? sqrt(ss / (3.0 * (double)a.d.vox())) : 0.0;
     }
-    const float inv_hi = (float)inv, inv_lo = isfinite(inv_hi) ? (float)(inv - (double)inv_hi) : 0.f;
+    const bool in_pairs = MODE == TC_UNPACK_C64 && inv >= 0x1p-100 && inv <= 0x1p100;
+    const float inv_hi = in_pairs ? (float)inv : 0.f, inv_lo = in_pairs ? (float)(inv - (double)inv_hi) : 0.f;
     uint32_t local = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++local) {
       // the abort flag is read once per warp so that all lanes leave together
@@ -340,8 +343,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) conv_tc_kernel(const __grid_con
           for (int c = 0; c < 3; ++c) {
             const float yr = acc[c] + bias[c], yi = acc[3 + c] + bias[3 + c];
             V vi = v[(size_t)c * V0 + vox];
-            if constexpr (MODE == TC_UNPACK_C64) {
-              if (isfinite(yr) && isfinite(yi) && isfinite(inv)) {
+            if (in_pairs) {
+              if (isfinite(yr) && isfinite(yi)) {
                 vi.x = add_scaled(vi.x, yr, inv_hi, inv_lo);
                 vi.y = add_scaled(vi.y, yi, inv_hi, inv_lo);
               } else {
