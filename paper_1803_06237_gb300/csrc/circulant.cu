@@ -750,8 +750,9 @@ __global__ void __launch_bounds__(256) to_tiles_kernel(const float2* __restrict_
 
 // x = P b, then L y = x and U z = y from the tile stream, one CTA per
 // frequency.  HBM-bound: the factors are read once.  A stage is up to four
-// tiles of one block row (16 KB); two stages are in flight (asynchronous
-// copies) while one is used, 32 KB a CTA, four CTAs an SM.  Warp w sums rows
+// tiles of one block row (16 KB); two stages, 32 KB a CTA, are in flight
+// (asynchronous copies) while one is used.  48 KB of stages and the vector: four
+// CTAs an SM up to 992 unknowns, three beyond.  Warp w sums rows
 // 4 w .. 4 w + 3 of a tile, a lane per column; at the end of a block row the
 // sums meet in shared memory and warp 0 solves the diagonal tile.  The rows
 // used to be read by seven threads each, 4 bytes at a time: 599 us for 396

@@ -1624,10 +1624,8 @@ static vie_status run_jm(vie_plan* p, const V* x, V* y, const V* ghat, const V* 
   vie_status st = launch_x<V>(true, 0, p->ax[0], pp, 1, nx, NL, NL, twx, mode, s, NL);
   if (st != VIE_OK) return st;
   PassBGeom g{ny, nz, NL, Mx, My, Mz, p->kf[1], p->kf[2]};
-  if (!done) {
-    st = launch_b_any<V>(pp, 1, g, 6, chat, p->kappa, twy, s, &done);
-    if (st != VIE_OK) return st;
-  }
+  st = launch_b_any<V>(pp, 1, g, 6, chat, p->kappa, twy, s, &done);
+  if (st != VIE_OK) return st;
   if (!done && smem_b <= 220 * 1024) {
     VIE_CUDA_TRY(allow_shared(pass_b_jm_kernel<V>, smem_b));
     pass_b_jm_kernel<V><<<(unsigned)Mx, 256, smem_b, s>>>((V*)p->jm_work, ghat, chat, g, radices_of(p->ax[1]),

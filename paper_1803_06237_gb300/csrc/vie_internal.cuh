@@ -194,8 +194,8 @@ struct vie_plan {
   void* jm_work = nullptr;    // 6 ny nz Mx complex128
   int jm_gen = -1;            // contrast generation the 6N contrast was built from
   int contrast_gen = 0;       // incremented whenever the contrast is set
-  int x_lpb = 0;              // forward x pass: > 0 four-step with that many lines per block,
-                              // < 0 three-factor with -x_lpb lines per block, 0 heuristic
+  int x_lpb = 0;              // forward x pass chosen by the tuner: 5 four-step, -5 three-factor (five lines
+                              // per block, where compiled), 0 the default
   int x_lpb_inv = 0;          // the same for the inverse x pass
   double tune_ms = 0.0;       // VIE_PLAN_AUTOTUNE host time
   int tune_candidates = 0;
