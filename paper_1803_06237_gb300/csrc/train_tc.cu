@@ -32,6 +32,7 @@
 // (160 x 40 x 11), most of it the ends of short kernels (a GEMM of 14 CTAs
 // with four chunks each takes 14 us, one of 152 with nine takes 22).
 #include <cuda_bf16.h>
+#include <limits.h>
 #include <stdio.h>
 
 #include "net.cuh"
@@ -61,11 +62,9 @@ struct DwLayer {
   int nxp, nxc;              // padded row, chunks per row
   int block0;                // first block of the operand launch
   int cta0, ctas;            // CTAs of the GEMM
-  int layer;                 // its maps
 };
 struct DwArgs {
-  DwLayer l[kNumLayers];     // the `count` layers of this group
-  int count;
+  DwLayer l[kNumLayers];     // the layers of this group; block0 and cta0 of the rest: none reaches them
   int stages;
   float* partial;            // [CTA][27][32][C], CTAs 27 x 32 x 32 apart
   int* bad;
@@ -82,7 +81,7 @@ struct DwArgs {
 __global__ void __launch_bounds__(256) dw_operands_kernel(const __grid_constant__ DwArgs args) {
   __shared__ __nv_bfloat16 t[kDwChunk + 2][33];
   __shared__ float bsum[8][33];
-  int li = args.count - 1;
+  int li = kNumLayers - 1;
   while (li > 0 && (int)blockIdx.x < args.l[li].block0) --li;
   const DwLayer& L = args.l[li];
   const Dims d = L.d;
@@ -260,13 +259,13 @@ constexpr size_t kDwPartial = (size_t)27 * 32 * 32;   // floats of a CTA's parti
 
 __global__ void __launch_bounds__(kDwThreads, 1) dw_tc_kernel(const __grid_constant__ DwMaps maps,
                                                               const __grid_constant__ DwArgs args) {
-  int li = args.count - 1;
+  int li = kNumLayers - 1;
   while (li > 0 && (int)blockIdx.x < args.l[li].cta0) --li;
   const DwLayer& L = args.l[li];
   const int cta = blockIdx.x - L.cta0;
   float* partial = args.partial + blockIdx.x * kDwPartial;
-  if (L.C == 32) dw_gemm<32>(maps.a[L.layer], maps.b[L.layer], L, cta, args.stages, partial, args.bad);
-  else dw_gemm<16>(maps.a[L.layer], maps.b[L.layer], L, cta, args.stages, partial, args.bad);
+  if (L.C == 32) dw_gemm<32>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
+  else dw_gemm<16>(maps.a[li], maps.b[li], L, cta, args.stages, partial, args.bad);
 }
 
 // gw[(o ci + c) 27 + t] += sum_b partial[b][t][o][c] over the layer's CTAs
@@ -615,13 +614,16 @@ static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, int 
   const __nv_bfloat16* in[kNumLayers] = {T->X, T->a[1], T->a[2], T->a[3], T->decin[2], T->decin[1], T->decin[0],
                                          T->u[0]};
   DwArgs a{};
-  a.count = l1 - l0;
+  DwMaps maps{};
+  const int count = l1 - l0;
   long chunks[kNumLayers], want = 0;
   unsigned blocks = 0;
-  for (int k = 0; k < a.count; ++k) {
+  for (int k = count; k < kNumLayers; ++k) a.l[k].block0 = a.l[k].cta0 = INT_MAX;
+  for (int k = 0; k < count; ++k) {
     const int l = l0 + k;
     DwLayer& L = a.l[k];
-    L.layer = l;
+    maps.a[k] = T->mP.a[l];
+    maps.b[k] = T->mP.b[l];
     L.d = T->L[kLayerLevel[l]];
     L.g = l == OUTL ? T->dY : T->dpre[l];
     L.in = in[l];
@@ -644,16 +646,16 @@ static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, int 
   // one CTA per SM at most, each layer's share by its chunks: one each, then
   // to the layer with the most chunks a CTA
   const int ctas = (int)(want < T->sms ? want : T->sms);
-  for (int k = 0; k < a.count; ++k) a.l[k].ctas = 1;
-  for (int n = a.count; n < ctas; ++n) {
+  for (int k = 0; k < count; ++k) a.l[k].ctas = 1;
+  for (int n = count; n < ctas; ++n) {
     int most = 0;
-    for (int k = 1; k < a.count; ++k)
+    for (int k = 1; k < count; ++k)
       if (chunks[k] * a.l[most].ctas > chunks[most] * a.l[k].ctas) most = k;
     if (a.l[most].ctas >= chunks[most]) break;
     ++a.l[most].ctas;
   }
   int used = 0;
-  for (int k = 0; k < a.count; ++k) {
+  for (int k = 0; k < count; ++k) {
     a.l[k].cta0 = used;
     used += a.l[k].ctas;
   }
@@ -672,9 +674,9 @@ static vie_status weight_grads_tc(const TcTrain* T, const TcTrainParams& P, int 
   dw_operands_kernel<<<blocks, 256, 0, s>>>(a);
   VIE_LAUNCH_CHECK();
   VIE_CUDA_TRY(cudaFuncSetAttribute(dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  dw_tc_kernel<<<used, kDwThreads, smem, s>>>(T->mP, a);
+  dw_tc_kernel<<<used, kDwThreads, smem, s>>>(maps, a);
   VIE_LAUNCH_CHECK();
-  dw_reduce_kernel<<<dim3((unsigned)(kDwPartial / 256), (unsigned)a.count, 8), 256, 0, s>>>(a);
+  dw_reduce_kernel<<<dim3((unsigned)(kDwPartial / 256), (unsigned)count, 8), 256, 0, s>>>(a);
   VIE_LAUNCH_CHECK();
   return VIE_OK;
 }
