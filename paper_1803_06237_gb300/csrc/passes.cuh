@@ -37,8 +37,8 @@ struct PassPtrs {
 // a pass starts ahead of the wait have landed before its blocks leave.
 template <typename V>
 __device__ __forceinline__ bool skip_after_wait(const PassPtrs<V>& pp) {
+  const int* f = pp.live[blockIdx.y];   // a kernel parameter
   pdl_wait();
-  const int* f = pp.live[blockIdx.y];
   if (f == nullptr || *(const volatile int*)f != 0) return false;
   __pipeline_commit();
   __pipeline_wait_prior(0);
