@@ -42,6 +42,7 @@ def test_no_pass_leaves_before_its_wait(name, kernels):
 def test_the_flag_is_read_behind_the_wait():
     text = _read("passes.cuh")
     body = _body(text, text.index("bool skip_after_wait"))
-    assert body.index("pdl_wait()") < body.index("pp.live")
+    assert body.index("pdl_wait()") < body.index("*(const volatile int*)f")
+    assert body.count("*f") == 0 and body.count("*(") == 1 and body.count("pp.live") == 1   # its only read
     for name in ("matvec.cu", "any_x.cuh", "any_b.cuh"):
         assert not re.search(r"pp\.live(?!\[k\] = )", _read(name)), name
